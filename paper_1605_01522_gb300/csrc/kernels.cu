@@ -1019,13 +1019,15 @@ struct KScaleConvert {
   }
 };
 
-// the same with a = 1 / sqrt(nrm2[0]) read from device memory (the norm of
-// the previous Arnoldi vector, so that a captured iteration graph normalises
-// its input itself); out may be null (in-place scaling only)
+// the same with a = inv[0] read from device memory (1 / |w| of the previous
+// Arnoldi vector, so that a captured iteration graph normalises its input
+// itself); out may be null (in-place scaling only).  The square root and the
+// division are done once, by the pass that made the norm: done here by every
+// thread they took 29 us of FP64 time on 1.37 M entries (5 us of memory traffic).
 template <typename TO>
-__device__ __forceinline__ void d_scale_convert_dev(double *__restrict__ v, const double *__restrict__ nrm2,
+__device__ __forceinline__ void d_scale_convert_dev(double *__restrict__ v, const double *__restrict__ inv,
                                                     TO *__restrict__ out, int64_t n, int bid_, int nb_) {
-  const double a = 1.0 / sqrt(nrm2[0]);
+  const double a = inv[0];
   for (int64_t i = (int64_t)bid_ * blockDim.x + threadIdx.x; i < n; i += (int64_t)nb_ * blockDim.x) {
     const double t = a * v[i];
     v[i] = t;
@@ -1037,12 +1039,12 @@ struct KScaleConvertDev {
   static constexpr int kMaxThreads = kThreads;
   struct Args {
     double *v;
-    const double *nrm2;
+    const double *inv;
     TO *out;
     int64_t n;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_scale_convert_dev<TO>(a.v, a.nrm2, a.out, a.n, bid, nb);
+    d_scale_convert_dev<TO>(a.v, a.inv, a.out, a.n, bid, nb);
   }
 };
 
@@ -1062,11 +1064,68 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   return s;  // valid in thread 0
 }
 
-constexpr int kTile = kThreads;  // rows of w staged per step
+constexpr int kTile = kThreads;  // entries of w staged per step
 constexpr int kMaxQ = 64;        // rows of V handled per launch (8 per warp)
+// Passes over at most this many CTAs are finished by their last CTA (their
+// partial sums added up there) instead of by a launch of k_reduce_partials.
+constexpr int kFinishBlocks = 304;
 
-// partial[q*nblk + b] = sum over chunk b of V_q[i] * ws[i] for the staged tile;
-// warp p owns rows q = p, p+8, ... and reads them coalesced.
+// Sum over the warp of each of a lane's 8 values: at offsets 16, 8, 4 a lane
+// keeps one half of its rows and adds the partner's half, then two ordinary
+// butterfly steps.  9 float64 adds per lane instead of the 40 of eight
+// butterflies (the adds go through the FP64 pipe, which bounds these passes).
+// Lane l holds the sum of row l >> 2.
+__device__ __forceinline__ double warp_sum8(const double (&a)[8], int lane) {
+  double b[4], c[2];
+  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    b[i] = (h16 ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, h16 ? a[i] : a[i + 4], 16);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    c[i] = (h8 ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, h8 ? b[i] : b[i + 2], 8);
+  double d = (h4 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h4 ? c[0] : c[1], 4);
+  d += __shfl_xor_sync(0xffffffffu, d, 2);
+  d += __shfl_xor_sync(0xffffffffu, d, 1);
+  return d;
+}
+
+// one warp: p[0] + ... + p[n - 1] (valid in every lane).  The partial sums
+// come from other CTAs of this launch or of the previous one: read from L2.
+__device__ __forceinline__ double warp_sum_partials(const double *p, int n, int lane) {
+  double a = 0.0;
+  for (int i = lane; i < n; i += 32) a += __ldcg(p + i);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+// The CTA of a pass that comes last (the counter says so, and is set back to
+// 0 for the next pass) adds up the nb partial sums of each of the k rows, in
+// the order of k_reduce_partials; with `inv` also out[k] = 1 / sqrt(out[0]).
+// Every thread of every CTA calls this after it has written its partials.
+__device__ __forceinline__ void finish_rows(const double *partial, int k, int nb, double *out, unsigned *cnt,
+                                            bool inv) {
+  __shared__ int last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(cnt, 1u) == (unsigned)(nb - 1) ? 1 : 0;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int q = warp; q < k; q += kThreads / 32) {
+    const double t = warp_sum_partials(partial + (int64_t)q * nb, nb, lane);
+    if (lane == 0) {
+      out[q] = t;
+      if (inv) out[k] = 1.0 / sqrt(t);
+    }
+  }
+  if (threadIdx.x == 0) *cnt = 0u;
+}
+
+// acc[m] += V_q[t0 ..] . ws over a staged tile for the warp's rows q = warp +
+// 8 m: a lane's 8 loads of a full tile are issued before the first product
 __device__ __forceinline__ void tile_dots(const double *__restrict__ V, int64_t ldv, int k, int64_t t0, int cnt,
                                           const double *ws, double (&acc)[kMaxQ / 8]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1074,47 +1133,55 @@ __device__ __forceinline__ void tile_dots(const double *__restrict__ V, int64_t 
   for (int m = 0; m < kMaxQ / 8; ++m) {
     const int q = warp + 8 * m;
     if (q < k) {
-      const double *vq = V + (int64_t)q * ldv + t0;
+      const double *vq = V + (int64_t)q * ldv + t0 + lane;
       double s = acc[m];  // one FMA chain per row across the tiles (no extra add per tile)
-      for (int t = lane; t < cnt; t += 32) s = fma(vq[t], ws[t], s);
+      if (cnt == kTile) {
+        double v[kTile / 32];
+#pragma unroll
+        for (int u = 0; u < kTile / 32; ++u) v[u] = vq[u * 32];
+#pragma unroll
+        for (int u = 0; u < kTile / 32; ++u) s = fma(v[u], ws[lane + u * 32], s);
+      } else {
+        for (int t = 0; t < cnt - lane; t += 32) s = fma(vq[t], ws[lane + t], s);
+      }
       acc[m] = s;
     }
   }
 }
 
-__device__ __forceinline__ void store_dots(int k, int nblk, double (&acc)[kMaxQ / 8], double *__restrict__ partial,
-                                           int bid) {
+__device__ __forceinline__ void store_dots(int k, int nblk, const double (&acc)[kMaxQ / 8],
+                                           double *__restrict__ partial, int bid) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int m = 0; m < kMaxQ / 8; ++m) {
-    const int q = warp + 8 * m;
-    if (q < k) {
-      double v = acc[m];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) partial[(int64_t)q * nblk + bid] = v;
-    }
-  }
+  const double t = warp_sum8(acc, lane);
+  const int q = warp + 8 * (lane >> 2);
+  if ((lane & 3) == 0 && q < k) partial[(int64_t)q * nblk + bid] = t;
+}
+
+// entries [lo, hi) of CTA bid: whole tiles, as even as possible
+__device__ __forceinline__ void tile_range(int64_t n, int nblk, int bid, int64_t &lo, int64_t &hi) {
+  const int64_t tiles = (n + kTile - 1) / kTile, per = (tiles + nblk - 1) / nblk;
+  lo = (int64_t)bid * per * kTile;
+  hi = min(n, lo + per * kTile);
 }
 
 // h_q = V_q . w for q < k (w may be one of the rows of V)
 __device__ __forceinline__ void d_mdot(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ w, int64_t n,
-       double *__restrict__ partial, int nblk, int bid_, int nb_) {
+       double *__restrict__ partial, int nblk, double *out, unsigned *cnt, int bid_) {
   __shared__ double ws[kTile];
-  const int64_t chunk = (n + nblk - 1) / nblk;
-  const int64_t lo = (int64_t)bid_ * chunk;
-  const int64_t hi = min(n, lo + chunk);
+  int64_t lo, hi;
+  tile_range(n, nblk, bid_, lo, hi);
   double acc[kMaxQ / 8];
 #pragma unroll
   for (int m = 0; m < kMaxQ / 8; ++m) acc[m] = 0.0;
   for (int64_t t0 = lo; t0 < hi; t0 += kTile) {
-    const int cnt = (int)min((int64_t)kTile, hi - t0);
-    ws[threadIdx.x] = threadIdx.x < cnt ? w[t0 + threadIdx.x] : 0.0;
+    const int cnt_t = (int)min((int64_t)kTile, hi - t0);
+    ws[threadIdx.x] = threadIdx.x < cnt_t ? w[t0 + threadIdx.x] : 0.0;
     __syncthreads();
-    tile_dots(V, ldv, k, t0, cnt, ws, acc);
+    tile_dots(V, ldv, k, t0, cnt_t, ws, acc);
     __syncthreads();
   }
   store_dots(k, nblk, acc, partial, bid_);
+  if (cnt != nullptr) finish_rows(partial, k, nblk, out, cnt, false);
 }
 struct KMdot {
   static constexpr int kMaxThreads = kThreads;
@@ -1126,41 +1193,67 @@ struct KMdot {
     int64_t n;
     double *partial;
     int nblk;
+    double *out;    // with cnt: the k sums, added up by the last CTA
+    unsigned *cnt;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_mdot(a.V, a.ldv, a.k, a.w, a.n, a.partial, a.nblk, bid, nb);
+    d_mdot(a.V, a.ldv, a.k, a.w, a.n, a.partial, a.nblk, a.out, a.cnt, bid);
   }
 };
 
+// sum_q V_q[i] h_q, 8 loads in flight
+__device__ __forceinline__ double col_dot(const double *__restrict__ V, int64_t ldv, int k, const double *hs,
+                                          int64_t i) {
+  const double *v = V + i;
+  double s = 0.0;  // (a chain started from w_i would wait for its load)
+  int q = 0;
+  for (; q + 8 <= k; q += 8) {
+    double t[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) t[u] = v[(int64_t)(q + u) * ldv];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) s = fma(t[u], hs[q + u], s);
+  }
+  if (q + 4 <= k) {
+    double t[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) t[u] = v[(int64_t)(q + u) * ldv];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s = fma(t[u], hs[q + u], s);
+    q += 4;
+  }
+  for (; q < k; ++q) s = fma(v[(int64_t)q * ldv], hs[q], s);
+  return s;
+}
+
 // w <- w - sum_q V_q h_q, then partial dots V_q . w_new (CGS2 second pass)
 __device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h, double *__restrict__ w,
-            int64_t n, double *__restrict__ partial, int nblk, int bid_, int nb_) {
+            int64_t n, double *__restrict__ partial, int nblk, double *out, unsigned *cnt, int bid_) {
   __shared__ double ws[kTile];
   __shared__ double hs[kMaxQ];
   for (int q = threadIdx.x; q < k; q += blockDim.x) hs[q] = h[q];
   __syncthreads();
-  const int64_t chunk = (n + nblk - 1) / nblk;
-  const int64_t lo = (int64_t)bid_ * chunk;
-  const int64_t hi = min(n, lo + chunk);
+  int64_t lo, hi;
+  tile_range(n, nblk, bid_, lo, hi);
   double acc[kMaxQ / 8];
 #pragma unroll
   for (int m = 0; m < kMaxQ / 8; ++m) acc[m] = 0.0;
   for (int64_t t0 = lo; t0 < hi; t0 += kTile) {
-    const int cnt = (int)min((int64_t)kTile, hi - t0);
+    const int cnt_t = (int)min((int64_t)kTile, hi - t0);
     double wn = 0.0;
-    if (threadIdx.x < cnt) {
+    if (threadIdx.x < cnt_t) {
       const int64_t i = t0 + threadIdx.x;
-      double s = 0.0;  // (a chain started from w_i would wait for its load)
-      for (int q = 0; q < k; ++q) s += V[(int64_t)q * ldv + i] * hs[q];
-      wn = w[i] - s;
+      const double wi = w[i];
+      wn = wi - col_dot(V, ldv, k, hs, i);
       w[i] = wn;
     }
     ws[threadIdx.x] = wn;
     __syncthreads();
-    tile_dots(V, ldv, k, t0, cnt, ws, acc);
+    tile_dots(V, ldv, k, t0, cnt_t, ws, acc);
     __syncthreads();
   }
   store_dots(k, nblk, acc, partial, bid_);
+  if (cnt != nullptr) finish_rows(partial, k, nblk, out, cnt, false);
 }
 struct KCgsFused {
   static constexpr int kMaxThreads = kThreads;
@@ -1173,23 +1266,22 @@ struct KCgsFused {
     int64_t n;
     double *partial;
     int nblk;
+    double *out;
+    unsigned *cnt;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_cgs_fused(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, bid, nb);
+    d_cgs_fused(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.out, a.cnt, bid);
   }
 };
 
-__device__ __forceinline__ void d_reduce_partials(const double *__restrict__ partial, int k, int nblk, double *__restrict__ out, int bid_, int nb_) {
-  __shared__ double sh[32];
+// out[q] = sum of the nblk partial sums of row q, one warp (CTA) per row
+__device__ __forceinline__ void d_reduce_partials(const double *__restrict__ partial, int k, int nblk, double *__restrict__ out, int bid_) {
   if (bid_ >= k) return;
-  const double *p = partial + (int64_t)bid_ * nblk;
-  double acc = 0.0;
-  for (int i = threadIdx.x; i < nblk; i += blockDim.x) acc += p[i];
-  const double s = block_sum(acc, sh);
+  const double s = warp_sum_partials(partial + (int64_t)bid_ * nblk, nblk, threadIdx.x);
   if (threadIdx.x == 0) out[bid_] = s;
 }
 struct KReducePartials {
-  static constexpr int kMaxThreads = kThreads;
+  static constexpr int kMaxThreads = 32;
   struct Args {
     const double *partial;
     int k;
@@ -1197,31 +1289,30 @@ struct KReducePartials {
     double *out;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_reduce_partials(a.partial, a.k, a.nblk, a.out, bid, nb);
+    d_reduce_partials(a.partial, a.k, a.nblk, a.out, bid);
   }
 };
 
+// w <- w - sum_q V_q h_q, then |w|^2 and 1 / |w| (last CTA)
 __device__ __forceinline__ void d_cgs_update(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h,
-             double *__restrict__ w, int64_t n, double *__restrict__ partial, int nblk, int bid_, int nb_) {
-  __shared__ double hs[64];
+             double *__restrict__ w, int64_t n, double *__restrict__ partial, int nblk, double *out, unsigned *cnt,
+             int bid_) {
+  __shared__ double hs[kMaxQ];
   __shared__ double sh[32];
   for (int q = threadIdx.x; q < k; q += blockDim.x) hs[q] = h[q];
   __syncthreads();
-  const int64_t chunk = (n + nblk - 1) / nblk;
-  const int64_t lo = (int64_t)bid_ * chunk;
-  const int64_t hi = min(n, lo + chunk);
+  int64_t lo, hi;
+  tile_range(n, nblk, bid_, lo, hi);
   double nrm = 0.0;
   for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-    double s = 0.0;  // (a chain started from w_i would wait for its load)
-    for (int q = 0; q < k; ++q) s += V[(int64_t)q * ldv + i] * hs[q];
-    const double wn = w[i] - s;
+    const double wi = w[i];
+    const double wn = wi - col_dot(V, ldv, k, hs, i);
     w[i] = wn;
     nrm += wn * wn;
   }
-  if (partial != nullptr) {
-    const double t = block_sum(nrm, sh);
-    if (threadIdx.x == 0) partial[bid_] = t;
-  }
+  const double t = block_sum(nrm, sh);
+  if (threadIdx.x == 0) partial[bid_] = t;
+  finish_rows(partial, 1, nblk, out, cnt, true);
 }
 struct KCgsUpdate {
   static constexpr int kMaxThreads = kThreads;
@@ -1234,9 +1325,11 @@ struct KCgsUpdate {
     int64_t n;
     double *partial;
     int nblk;
+    double *out;
+    unsigned *cnt;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_cgs_update(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, bid, nb);
+    d_cgs_update(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.out, a.cnt, bid);
   }
 };
 
@@ -1797,9 +1890,9 @@ void scale_convert(double *v, double a, TO *out, int64_t n, cudaStream_t s) {
 template void scale_convert<float>(double *, double, float *, int64_t, cudaStream_t);
 template void scale_convert<double>(double *, double, double *, int64_t, cudaStream_t);
 template <typename TO>
-void scale_convert_dev(double *v, const double *nrm2, TO *out, int64_t n, cudaStream_t s) {
+void scale_convert_dev(double *v, const double *inv, TO *out, int64_t n, cudaStream_t s) {
   HookScope hs(s, K_VECTOR, (16.0 + (out ? sizeof(TO) : 0)) * n, 8, n, (double)n);
-  if (n) go<KScaleConvertDev<TO>>(ew_grid(n), kThreads, 0, s, {v, nrm2, out, n});
+  if (n) go<KScaleConvertDev<TO>>(ew_grid(n), kThreads, 0, s, {v, inv, out, n});
 }
 template void scale_convert_dev<float>(double *, const double *, float *, int64_t, cudaStream_t);
 template void scale_convert_dev<double>(double *, const double *, double *, int64_t, cudaStream_t);
@@ -1809,43 +1902,46 @@ void scale(const double *x, double a, double *y, int64_t n, cudaStream_t s) {
   if (n) go<KScale>(ew_grid(n), kThreads, 0, s, {x, a, y, n});
 }
 
-// CTAs of the CGS2 passes over a length-n basis: one per 2048 entries, up
-// to four per SM; small systems (below 32 k entries) take up to 16, one
-// staged tile of w (kTile entries) each at least, so that their passes do
-// not loop over tiles in one or two CTAs.  (More CTAs for mid-size systems
-// would help a system solved alone but slow down batches, whose merged
-// launches fill the GPU already; the count is per system, so a batch and a
-// solo solve reduce in the same order.)
+// CTAs of the CGS2 passes over a length-n basis: whole tiles of kTile
+// entries, one per CTA up to four CTAs per SM, then as many tiles per CTA as
+// that takes.  (The count is per system, so a batch and a solo solve reduce
+// in the same order.)
 int mdot_blocks(int64_t n) {
-  int64_t b = n / 2048;
-  b = std::max(b, std::min<int64_t>((n + kTile - 1) / kTile, 16));
-  if (b < 1) b = 1;
-  if (b > 152 * 4) b = 152 * 4;
-  return (int)b;
+  const int64_t tiles = std::max<int64_t>(1, (n + kTile - 1) / kTile);
+  const int64_t per = (tiles + 152 * 4 - 1) / (152 * 4);
+  return (int)((tiles + per - 1) / per);
 }
 
 void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, double *partial, int nblk,
-          cudaStream_t s) {
-  HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 1), 1, n, 2.0 * n * k);
-  go<KMdot>(nblk, kThreads, 0, s, {V, ldv, k, w, n, partial, nblk});
+          cudaStream_t s, double *out, unsigned *cnt) {
+  if (nblk > kFinishBlocks) cnt = nullptr;
+  {
+    HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 1), 1, n, 2.0 * n * k);
+    go<KMdot>(nblk, kThreads, 0, s, {V, ldv, k, w, n, partial, nblk, out, cnt});
+  }
+  if (out && !cnt) reduce_partials(partial, k, nblk, out, s);
 }
 
 void reduce_partials(const double *partial, int k, int nblk, double *out, cudaStream_t s) {
   HookScope hs(s, K_ARNOLDI, 8.0 * (double)k * nblk, 2, k, (double)k * nblk);
   // recorded launches take a grid that does not depend on k (blocks >= k return)
-  go<KReducePartials>(g_rec ? (unsigned)kMaxQ : (unsigned)k, kThreads, 0, s, {partial, k, nblk, out});
+  go<KReducePartials>(g_rec ? (unsigned)kMaxQ : (unsigned)k, 32, 0, s, {partial, k, nblk, out});
 }
 
 void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
-               int nblk, cudaStream_t s) {
-  HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 3, n, 4.0 * n * k);
-  go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk});
+               int nblk, double *out, unsigned *cnt, cudaStream_t s) {
+  if (nblk > kFinishBlocks) cnt = nullptr;
+  {
+    HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 3, n, 4.0 * n * k);
+    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, out, cnt});
+  }
+  if (!cnt) reduce_partials(partial, k, nblk, out, s);
 }
 
 void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
-                double *partial, int nblk, cudaStream_t s) {
+                double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s) {
   HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 4, n, 2.0 * n * k + 2.0 * n);
-  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk});
+  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, out, cnt});
 }
 
 void gemv_add(const double *Z, int64_t ldz, int k, const double *y, double *x, int64_t n, cudaStream_t s) {

@@ -203,21 +203,27 @@ template <typename TI, typename TO> void convert(const TI *in, TO *out, int64_t 
 void scale(const double *x, double a, double *y, int64_t n, cudaStream_t s);                      // y = a x
 // v = a v and out = (TO) v in one pass
 template <typename TO> void scale_convert(double *v, double a, TO *out, int64_t n, cudaStream_t s);
-// the same with a = 1 / sqrt(nrm2[0]) taken from device memory; out may be null
+// the same with a = inv[0] taken from device memory; out may be null
 template <typename TO>
-void scale_convert_dev(double *v, const double *nrm2, TO *out, int64_t n, cudaStream_t s);
+void scale_convert_dev(double *v, const double *inv, TO *out, int64_t n, cudaStream_t s);
 
 // Arnoldi (float64).  V holds k row vectors of length n, row q at V + q*ldv.
+// partial: k * nblk doubles of scratch, nblk = mdot_blocks(n); out: device
+// memory; cnt: a device counter that is 0 between passes (passes over few
+// CTAs add up their partial sums in their last CTA, the others launch
+// reduce_partials; the order of the sums is the same).
 int mdot_blocks(int64_t n);
+// out[q] = V_q . w; with out null only partial[q*nblk+b], for a later
+// reduce_partials; cnt may be null
 void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, double *partial,
-          int nblk, cudaStream_t s);                                   // partial[q*nblk+b]
+          int nblk, cudaStream_t s, double *out = nullptr, unsigned *cnt = nullptr);
 void reduce_partials(const double *partial, int k, int nblk, double *out, cudaStream_t s);
-// w -= sum_q V_q h_q and partial dots V_q . w_new in one pass (k <= 64)
+// w -= sum_q V_q h_q and out[q] = V_q . w_new in one pass (k <= 64)
 void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
-               int nblk, cudaStream_t s);
-// w -= sum_q V_q h_q; if partial != null also partial[b] = sum w_new^2 over block b
+               int nblk, double *out, unsigned *cnt, cudaStream_t s);
+// w -= sum_q V_q h_q, out[0] = |w_new|^2, out[1] = 1 / |w_new|
 void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
-                double *partial, int nblk, cudaStream_t s);
+                double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s);
 // x += sum_q Z_q y_q
 void gemv_add(const double *Z, int64_t ldz, int k, const double *y, double *x, int64_t n,
               cudaStream_t s);

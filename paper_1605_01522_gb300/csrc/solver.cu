@@ -1139,6 +1139,7 @@ struct mfs_handle {
   int m = 0, nblk = 1;
   double *V = nullptr, *Z = nullptr, *xd = nullptr, *bd = nullptr, *rd = nullptr, *partial = nullptr;
   double *hdev = nullptr, *ydev = nullptr;
+  unsigned *cnt = nullptr;  // CTAs done in the running Arnoldi pass (0 between passes)
   float *in32 = nullptr, *out32 = nullptr;
   // hdev / hpin: the Arnoldi sums of iterations of even and odd Krylov index
   // at 0 and 256 (136 each), a dot product at kDotSlot
@@ -1205,8 +1206,7 @@ void precond_apply(mfs_handle *h, const double *v, double *z, bool staged = fals
 
 // ||x||^2 of n doubles, deterministic, result in host memory
 double dot_host(mfs_handle *h, const double *x, const double *y) {
-  dev::mdot(x, 0, 1, y, h->n, h->partial, h->nblk, h->s);
-  dev::reduce_partials(h->partial, 1, h->nblk, h->hdev + kDotSlot, h->s);
+  dev::mdot(x, 0, 1, y, h->n, h->partial, h->nblk, h->s, h->hdev + kDotSlot, h->cnt);
   MFS_CUDA(cudaMemcpyAsync(h->hpin + kDotSlot, h->hdev + kDotSlot, sizeof(double), cudaMemcpyDeviceToHost, h->s));
   dev::pdl_break();
   MFS_CUDA(cudaStreamSynchronize(h->s));
@@ -1263,7 +1263,8 @@ struct KrylovLS {
     jend = 0;
   }
   // column j from the Arnoldi sums hp (h1 at [0, j], |w|^2 before the
-  // projections at [j + 1], h2 at [64, 64 + j], |w|^2 after at [128]);
+  // projections at [j + 1], h2 at [64, 64 + j], |w|^2 after at [128], 1 / |w|
+  // at [129]);
   // false when a sum is not finite
   bool column(const double *hp, int j) {
     const double nw0 = std::sqrt(hp[j + 1]);
@@ -1309,12 +1310,9 @@ struct KrylovLS {
 void arnoldi(mfs_handle *h, int j, double *w, double *hd, cudaStream_t s) {
   const int64_t n = h->n;
   // CGS2: h1 = V^T w (and |w|^2), w -= V h1, h2 = V^T w, w -= V h2 (and |w|^2)
-  dev::mdot(h->V, n, j + 2, w, n, h->partial, h->nblk, s);
-  dev::reduce_partials(h->partial, j + 2, h->nblk, hd, s);
-  dev::cgs_fused(h->V, n, j + 1, hd, w, n, h->partial, h->nblk, s);
-  dev::reduce_partials(h->partial, j + 1, h->nblk, hd + 64, s);
-  dev::cgs_update(h->V, n, j + 1, hd + 64, w, n, h->partial, h->nblk, s);
-  dev::reduce_partials(h->partial, 1, h->nblk, hd + 128, s);
+  dev::mdot(h->V, n, j + 2, w, n, h->partial, h->nblk, s, hd, h->cnt);
+  dev::cgs_fused(h->V, n, j + 1, hd, w, n, h->partial, h->nblk, hd + 64, h->cnt, s);
+  dev::cgs_update(h->V, n, j + 1, hd + 64, w, n, h->partial, h->nblk, hd + 128, h->cnt, s);
 }
 
 // Solves and other solve-phase calls (apply, matvec) running in this process.
@@ -1382,9 +1380,9 @@ int fgmres(mfs_handle *h, const double *b, double *x, double tol, mfs_info *info
     double *w = h->V + (int64_t)(j + 1) * n;
     auto body = [&]() {
       if (j > 0) {
-        const double *nrm2 = hdb[(j - 1) & 1] + 128;
-        if (h->p32) dev::scale_convert_dev<float>(vj, nrm2, h->in32, n, s);
-        else dev::scale_convert_dev<double>(vj, nrm2, nullptr, n, s);
+        const double *inv = hdb[(j - 1) & 1] + 129;
+        if (h->p32) dev::scale_convert_dev<float>(vj, inv, h->in32, n, s);
+        else dev::scale_convert_dev<double>(vj, inv, nullptr, n, s);
       }
       precond_apply(h, vj, zj, j > 0);
       matvec(h, zj, w);
@@ -1853,8 +1851,7 @@ static void fused_solve(FusedBatch &B, const double *const *rhs, double *const *
       matvec(h, xx[k], h->rd);
       dev::axpy<double>(h->rd, b[k], -1.0, h->n, s);
       dev::scale(h->rd, -1.0, h->rd, h->n, s);
-      dev::mdot(h->rd, 0, 1, h->rd, h->n, h->partial, h->nblk, s);
-      dev::reduce_partials(h->partial, 1, h->nblk, B.sums(k) + 132, s);
+      dev::mdot(h->rd, 0, 1, h->rd, h->n, h->partial, h->nblk, s, B.sums(k) + 132, h->cnt);
     }
     MFS_CUDA(cudaMemcpyAsync(B.hbpin, B.hb, (size_t)136 * ns * sizeof(double), cudaMemcpyDeviceToHost, s));
     MFS_CUDA(cudaStreamSynchronize(s));
@@ -2431,6 +2428,7 @@ void alloc_solver_work(mfs_handle *h) {
   h->partial = h->ar.zeros<double>((int64_t)64 * h->nblk);
   h->hdev = h->ar.zeros<double>(kHostSlots);
   h->ydev = h->ar.zeros<double>(64);
+  h->cnt = h->ar.zeros<unsigned>(1);
   if (h->prm.precision == MFS_FP32P) {
     h->in32 = h->ar.zeros<float>(h->n);
     h->out32 = h->ar.zeros<float>(h->n);

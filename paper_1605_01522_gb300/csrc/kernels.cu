@@ -1048,6 +1048,7 @@ struct KScaleConvertDev {
   }
 };
 
+// sum of v over the CTA (kThreads threads), valid in thread 0
 __device__ __forceinline__ double block_sum(double v, double *sh) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -1057,75 +1058,91 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
   __syncthreads();
   double s = 0.0;
   if (threadIdx.x < 32) {
-    s = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
+    s = l < kThreads / 32 ? sh[l] : 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    for (int o = kThreads / 64; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   }
-  return s;  // valid in thread 0
+  return s;
 }
 
-constexpr int kTile = kThreads;  // entries of w staged per step
+// The CGS2 passes over V (k rows of length n) and w.  The FP64 pipe bounds
+// them (a warp's float64 instruction takes 64 cycles of an SM quarter; HBM
+// delivers 1.6 times what the pipe can use), on small systems through the SM
+// with the most entries: so the entries are spread over all SMs in tiles of
+// 256 (arnoldi_plan) and the sums over lanes are kept short
+// (warp_sum_rows).  The three passes and their reductions at 23 rows, in a
+// graph: 48,510 entries 27 us (107 us with n / 2048 CTAs), 344,605 73 us
+// (133), 1.37 M 266 us (287; float64 floor 238).  Smaller tiles shared by
+// several threads an entry gained 4 us at 3,267 entries but cost a batch
+// of 96 such systems 9 % and were dropped.
+constexpr int kTile = kThreads;  // entries of w per step of a CTA
 constexpr int kMaxQ = 64;        // rows of V handled per launch (8 per warp)
-// Passes over at most this many CTAs are finished by their last CTA (their
-// partial sums added up there) instead of by a launch of k_reduce_partials.
-constexpr int kFinishBlocks = 304;
 
-// Sum over the warp of each of a lane's 8 values: at offsets 16, 8, 4 a lane
-// keeps one half of its rows and adds the partner's half, then two ordinary
-// butterfly steps.  9 float64 adds per lane instead of the 40 of eight
-// butterflies (the adds go through the FP64 pipe, which bounds these passes).
-// Lane l holds the sum of row l >> 2.
-__device__ __forceinline__ double warp_sum8(const double (&a)[8], int lane) {
-  double b[4], c[2];
+// Sum over the warp of each of a lane's 8 values (HALF: only the first 4 are
+// used): at offsets 16, 8, 4 a lane keeps one half of its rows and adds the
+// partner's half, then two ordinary butterfly steps.  9 (6) float64 adds per
+// lane instead of the 40 of eight butterflies.  Lane l holds the sum of row
+// l >> 2 (HALF: l >> 3).
+template <bool HALF>
+__device__ __forceinline__ double warp_sum_rows(const double (&a)[8], int lane) {
   const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0, h4 = (lane & 4) != 0;
+  double c[2], d;
+  if constexpr (HALF) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    b[i] = (h16 ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, h16 ? a[i] : a[i + 4], 16);
+    for (int i = 0; i < 2; ++i)
+      c[i] = (h16 ? a[i + 2] : a[i]) + __shfl_xor_sync(0xffffffffu, h16 ? a[i] : a[i + 2], 16);
+    d = (h8 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h8 ? c[0] : c[1], 8);
+    d += __shfl_xor_sync(0xffffffffu, d, 4);
+  } else {
+    double b[4];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-    c[i] = (h8 ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, h8 ? b[i] : b[i + 2], 8);
-  double d = (h4 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h4 ? c[0] : c[1], 4);
+    for (int i = 0; i < 4; ++i)
+      b[i] = (h16 ? a[i + 4] : a[i]) + __shfl_xor_sync(0xffffffffu, h16 ? a[i] : a[i + 4], 16);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      c[i] = (h8 ? b[i + 2] : b[i]) + __shfl_xor_sync(0xffffffffu, h8 ? b[i] : b[i + 2], 8);
+    d = (h4 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h4 ? c[0] : c[1], 4);
+  }
   d += __shfl_xor_sync(0xffffffffu, d, 2);
   d += __shfl_xor_sync(0xffffffffu, d, 1);
   return d;
 }
 
-// one warp: p[0] + ... + p[n - 1] (valid in every lane).  The partial sums
-// come from other CTAs of this launch or of the previous one: read from L2.
-__device__ __forceinline__ double warp_sum_partials(const double *p, int n, int lane) {
+// p[0] + ... + p[n - 1] by the whole CTA, valid in thread 0.  The partial
+// sums come from other CTAs of this launch or of the previous one: read from L2.
+__device__ __forceinline__ double cta_sum_partials(const double *p, int n, double *sh) {
   double a = 0.0;
-  for (int i = lane; i < n; i += 32) a += __ldcg(p + i);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-  return a;
+  for (int i = threadIdx.x; i < n; i += kThreads) a += __ldcg(p + i);
+  return block_sum(a, sh);
 }
 
-// The CTA of a pass that comes last (the counter says so, and is set back to
-// 0 for the next pass) adds up the nb partial sums of each of the k rows, in
-// the order of k_reduce_partials; with `inv` also out[k] = 1 / sqrt(out[0]).
-// Every thread of every CTA calls this after it has written its partials.
-__device__ __forceinline__ void finish_rows(const double *partial, int k, int nb, double *out, unsigned *cnt,
-                                            bool inv) {
+// Passes with one result: the CTA that comes last (the counter says so, and
+// is set back to 0 for the next pass) adds up the nb partial sums, in the
+// order of k_reduce_partials: out[0], and with `inv` out[1] = 1 / sqrt(out[0]).
+// Every thread of every CTA calls this after thread 0 has written its
+// partial.  (For k results this would run k nb / 32 float64 warp
+// instructions on one SM: with 23 rows of 270 partials 3.8 us more than the
+// launch of k CTAs that it saves, with 13 partials 1.5 us.)
+__device__ __forceinline__ void finish_sum(const double *partial, int nb, double *out, unsigned *cnt, bool inv,
+                                           double *sh) {
   __shared__ int last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(cnt, 1u) == (unsigned)(nb - 1) ? 1 : 0;
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(cnt, 1u) == (unsigned)(nb - 1) ? 1 : 0;
+  }
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int q = warp; q < k; q += kThreads / 32) {
-    const double t = warp_sum_partials(partial + (int64_t)q * nb, nb, lane);
-    if (lane == 0) {
-      out[q] = t;
-      if (inv) out[k] = 1.0 / sqrt(t);
-    }
+  const double t = cta_sum_partials(partial, nb, sh);
+  if (threadIdx.x == 0) {
+    out[0] = t;
+    if (inv) out[1] = 1.0 / sqrt(t);
+    *cnt = 0u;
   }
-  if (threadIdx.x == 0) *cnt = 0u;
 }
 
 // acc[m] += V_q[t0 ..] . ws over a staged tile for the warp's rows q = warp +
-// 8 m: a lane's 8 loads of a full tile are issued before the first product
+// 8 m, a lane's 8 loads issued before the first product
 __device__ __forceinline__ void tile_dots(const double *__restrict__ V, int64_t ldv, int k, int64_t t0, int cnt,
                                           const double *ws, double (&acc)[kMaxQ / 8]) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1134,16 +1151,16 @@ __device__ __forceinline__ void tile_dots(const double *__restrict__ V, int64_t 
     const int q = warp + 8 * m;
     if (q < k) {
       const double *vq = V + (int64_t)q * ldv + t0 + lane;
-      double s = acc[m];  // one FMA chain per row across the tiles (no extra add per tile)
+      double v[kTile / 32], s = acc[m];  // one FMA chain per row across the tiles
       if (cnt == kTile) {
-        double v[kTile / 32];
 #pragma unroll
-        for (int u = 0; u < kTile / 32; ++u) v[u] = vq[u * 32];
-#pragma unroll
-        for (int u = 0; u < kTile / 32; ++u) s = fma(v[u], ws[lane + u * 32], s);
+        for (int u = 0; u < kTile / 32; ++u) v[u] = vq[32 * u];
       } else {
-        for (int t = 0; t < cnt - lane; t += 32) s = fma(vq[t], ws[lane + t], s);
+#pragma unroll
+        for (int u = 0; u < kTile / 32; ++u) v[u] = lane + 32 * u < cnt ? vq[32 * u] : 0.0;
       }
+#pragma unroll
+      for (int u = 0; u < kTile / 32; ++u) s = fma(v[u], ws[lane + 32 * u], s);
       acc[m] = s;
     }
   }
@@ -1152,54 +1169,21 @@ __device__ __forceinline__ void tile_dots(const double *__restrict__ V, int64_t 
 __device__ __forceinline__ void store_dots(int k, int nblk, const double (&acc)[kMaxQ / 8],
                                            double *__restrict__ partial, int bid) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const double t = warp_sum8(acc, lane);
-  const int q = warp + 8 * (lane >> 2);
-  if ((lane & 3) == 0 && q < k) partial[(int64_t)q * nblk + bid] = t;
-}
-
-// entries [lo, hi) of CTA bid: whole tiles, as even as possible
-__device__ __forceinline__ void tile_range(int64_t n, int nblk, int bid, int64_t &lo, int64_t &hi) {
-  const int64_t tiles = (n + kTile - 1) / kTile, per = (tiles + nblk - 1) / nblk;
-  lo = (int64_t)bid * per * kTile;
-  hi = min(n, lo + per * kTile);
-}
-
-// h_q = V_q . w for q < k (w may be one of the rows of V)
-__device__ __forceinline__ void d_mdot(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ w, int64_t n,
-       double *__restrict__ partial, int nblk, double *out, unsigned *cnt, int bid_) {
-  __shared__ double ws[kTile];
-  int64_t lo, hi;
-  tile_range(n, nblk, bid_, lo, hi);
-  double acc[kMaxQ / 8];
-#pragma unroll
-  for (int m = 0; m < kMaxQ / 8; ++m) acc[m] = 0.0;
-  for (int64_t t0 = lo; t0 < hi; t0 += kTile) {
-    const int cnt_t = (int)min((int64_t)kTile, hi - t0);
-    ws[threadIdx.x] = threadIdx.x < cnt_t ? w[t0 + threadIdx.x] : 0.0;
-    __syncthreads();
-    tile_dots(V, ldv, k, t0, cnt_t, ws, acc);
-    __syncthreads();
+  if (warp >= k) return;  // no rows
+  int q;
+  double t;
+  bool own;
+  if (k <= kMaxQ / 2) {
+    t = warp_sum_rows<true>(acc, lane);
+    q = warp + 8 * (lane >> 3);
+    own = (lane & 7) == 0;
+  } else {
+    t = warp_sum_rows<false>(acc, lane);
+    q = warp + 8 * (lane >> 2);
+    own = (lane & 3) == 0;
   }
-  store_dots(k, nblk, acc, partial, bid_);
-  if (cnt != nullptr) finish_rows(partial, k, nblk, out, cnt, false);
+  if (own && q < k) partial[(int64_t)q * nblk + bid] = t;
 }
-struct KMdot {
-  static constexpr int kMaxThreads = kThreads;
-  struct Args {
-    const double *V;
-    int64_t ldv;
-    int k;
-    const double *w;
-    int64_t n;
-    double *partial;
-    int nblk;
-    double *out;    // with cnt: the k sums, added up by the last CTA
-    unsigned *cnt;
-  };
-  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_mdot(a.V, a.ldv, a.k, a.w, a.n, a.partial, a.nblk, a.out, a.cnt, bid);
-  }
-};
 
 // sum_q V_q[i] h_q, 8 loads in flight
 __device__ __forceinline__ double col_dot(const double *__restrict__ V, int64_t ldv, int k, const double *hs,
@@ -1214,34 +1198,73 @@ __device__ __forceinline__ double col_dot(const double *__restrict__ V, int64_t 
 #pragma unroll
     for (int u = 0; u < 8; ++u) s = fma(t[u], hs[q + u], s);
   }
-  if (q + 4 <= k) {
-    double t[4];
+  double t[7];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) t[u] = v[(int64_t)(q + u) * ldv];
+  for (int u = 0; u < 7; ++u) t[u] = q + u < k ? v[(int64_t)(q + u) * ldv] : 0.0;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) s = fma(t[u], hs[q + u], s);
-    q += 4;
-  }
-  for (; q < k; ++q) s = fma(v[(int64_t)q * ldv], hs[q], s);
+  for (int u = 0; u < 7; ++u)
+    if (q + u < k) s = fma(t[u], hs[q + u], s);
   return s;
 }
 
+// h_q = V_q . w for q < k (w may be one of the rows of V)
+__device__ __forceinline__ void d_mdot(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ w, int64_t n,
+       double *__restrict__ partial, int nblk, int64_t per, double *out, unsigned *cnt, int bid_) {
+  __shared__ double ws[2][kTile];
+  __shared__ double sh[32];
+  const int64_t lo = (int64_t)bid_ * per, hi = min(n, lo + per);
+  double acc[kMaxQ / 8];
+#pragma unroll
+  for (int m = 0; m < kMaxQ / 8; ++m) acc[m] = 0.0;
+  // the next tile's w is loaded while this one is worked on; two buffers, so
+  // that one barrier a tile is enough
+  double wn = lo + threadIdx.x < hi ? w[lo + threadIdx.x] : 0.0;
+  int buf = 0;
+  for (int64_t t0 = lo; t0 < hi; t0 += kTile, buf ^= 1) {
+    const int c = (int)min((int64_t)kTile, hi - t0);
+    ws[buf][threadIdx.x] = wn;
+    const int64_t nx = t0 + kTile + threadIdx.x;
+    wn = nx < hi ? w[nx] : 0.0;
+    __syncthreads();
+    tile_dots(V, ldv, k, t0, c, ws[buf], acc);
+  }
+  store_dots(k, nblk, acc, partial, bid_);
+  if (cnt != nullptr) finish_sum(partial, nblk, out, cnt, false, sh);
+}
+struct KMdot {
+  static constexpr int kMaxThreads = kThreads;
+  struct Args {
+    const double *V;
+    int64_t ldv;
+    int k;
+    const double *w;
+    int64_t n;
+    double *partial;
+    int nblk;
+    int64_t per;    // entries per CTA
+    double *out;    // with cnt (k = 1): the sum, added up by the last CTA
+    unsigned *cnt;
+  };
+  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
+    d_mdot(a.V, a.ldv, a.k, a.w, a.n, a.partial, a.nblk, a.per, a.out, a.cnt, bid);
+  }
+};
+
 // w <- w - sum_q V_q h_q, then partial dots V_q . w_new (CGS2 second pass)
 __device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h, double *__restrict__ w,
-            int64_t n, double *__restrict__ partial, int nblk, double *out, unsigned *cnt, int bid_) {
+            int64_t n, double *__restrict__ partial, int nblk, int64_t per, int bid_) {
   __shared__ double ws[kTile];
   __shared__ double hs[kMaxQ];
   for (int q = threadIdx.x; q < k; q += blockDim.x) hs[q] = h[q];
   __syncthreads();
-  int64_t lo, hi;
-  tile_range(n, nblk, bid_, lo, hi);
+  const int64_t lo = (int64_t)bid_ * per, hi = min(n, lo + per);
   double acc[kMaxQ / 8];
 #pragma unroll
   for (int m = 0; m < kMaxQ / 8; ++m) acc[m] = 0.0;
   for (int64_t t0 = lo; t0 < hi; t0 += kTile) {
-    const int cnt_t = (int)min((int64_t)kTile, hi - t0);
+    const int c = (int)min((int64_t)kTile, hi - t0);
     double wn = 0.0;
-    if (threadIdx.x < cnt_t) {
+    if (threadIdx.x < c) {
       const int64_t i = t0 + threadIdx.x;
       const double wi = w[i];
       wn = wi - col_dot(V, ldv, k, hs, i);
@@ -1249,11 +1272,10 @@ __device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_
     }
     ws[threadIdx.x] = wn;
     __syncthreads();
-    tile_dots(V, ldv, k, t0, cnt_t, ws, acc);
+    tile_dots(V, ldv, k, t0, c, ws, acc);
     __syncthreads();
   }
   store_dots(k, nblk, acc, partial, bid_);
-  if (cnt != nullptr) finish_rows(partial, k, nblk, out, cnt, false);
 }
 struct KCgsFused {
   static constexpr int kMaxThreads = kThreads;
@@ -1266,22 +1288,22 @@ struct KCgsFused {
     int64_t n;
     double *partial;
     int nblk;
-    double *out;
-    unsigned *cnt;
+    int64_t per;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_cgs_fused(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.out, a.cnt, bid);
+    d_cgs_fused(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.per, bid);
   }
 };
 
-// out[q] = sum of the nblk partial sums of row q, one warp (CTA) per row
+// out[q] = sum of the nblk partial sums of row q, one CTA per row
 __device__ __forceinline__ void d_reduce_partials(const double *__restrict__ partial, int k, int nblk, double *__restrict__ out, int bid_) {
+  __shared__ double sh[32];
   if (bid_ >= k) return;
-  const double s = warp_sum_partials(partial + (int64_t)bid_ * nblk, nblk, threadIdx.x);
+  const double s = cta_sum_partials(partial + (int64_t)bid_ * nblk, nblk, sh);
   if (threadIdx.x == 0) out[bid_] = s;
 }
 struct KReducePartials {
-  static constexpr int kMaxThreads = 32;
+  static constexpr int kMaxThreads = kThreads;
   struct Args {
     const double *partial;
     int k;
@@ -1295,24 +1317,23 @@ struct KReducePartials {
 
 // w <- w - sum_q V_q h_q, then |w|^2 and 1 / |w| (last CTA)
 __device__ __forceinline__ void d_cgs_update(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h,
-             double *__restrict__ w, int64_t n, double *__restrict__ partial, int nblk, double *out, unsigned *cnt,
-             int bid_) {
+             double *__restrict__ w, int64_t n, double *__restrict__ partial, int nblk, int64_t per, double *out,
+             unsigned *cnt, int bid_) {
   __shared__ double hs[kMaxQ];
   __shared__ double sh[32];
   for (int q = threadIdx.x; q < k; q += blockDim.x) hs[q] = h[q];
   __syncthreads();
-  int64_t lo, hi;
-  tile_range(n, nblk, bid_, lo, hi);
+  const int64_t lo = (int64_t)bid_ * per, hi = min(n, lo + per);
   double nrm = 0.0;
-  for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) {
+  for (int64_t i = lo + threadIdx.x; i < hi; i += kTile) {
     const double wi = w[i];
     const double wn = wi - col_dot(V, ldv, k, hs, i);
     w[i] = wn;
-    nrm += wn * wn;
+    nrm = fma(wn, wn, nrm);
   }
   const double t = block_sum(nrm, sh);
   if (threadIdx.x == 0) partial[bid_] = t;
-  finish_rows(partial, 1, nblk, out, cnt, true);
+  finish_sum(partial, nblk, out, cnt, true, sh);
 }
 struct KCgsUpdate {
   static constexpr int kMaxThreads = kThreads;
@@ -1325,11 +1346,12 @@ struct KCgsUpdate {
     int64_t n;
     double *partial;
     int nblk;
+    int64_t per;
     double *out;
     unsigned *cnt;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_cgs_update(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.out, a.cnt, bid);
+    d_cgs_update(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.per, a.out, a.cnt, bid);
   }
 };
 
@@ -1902,22 +1924,44 @@ void scale(const double *x, double a, double *y, int64_t n, cudaStream_t s) {
   if (n) go<KScale>(ew_grid(n), kThreads, 0, s, {x, a, y, n});
 }
 
-// CTAs of the CGS2 passes over a length-n basis: whole tiles of kTile
-// entries, one per CTA up to four CTAs per SM, then as many tiles per CTA as
-// that takes.  (The count is per system, so a batch and a solo solve reduce
-// in the same order.)
-int mdot_blocks(int64_t n) {
+// CTAs of the CGS2 passes over a length-n basis and entries (whole tiles)
+// per CTA.  The SM with the most work sets the time: per CTA the three passes
+// run 32 float64 warp instructions a tile and row (768 at 24 rows, the middle
+// of a 50-column cycle), and its sums over lanes and its launch cost as much
+// as 120 such instructions (fitted to timings of 972 to 1.37 M entries).
+// More than two tiles per CTA only with 3 CTAs per SM, which hide the load
+// latency (1.37 M entries, 47 rows: 2 per SM 597 us, 3 per SM 500 us).
+// (The plan is per system, so a batch and a solo solve reduce in the same order.)
+struct ArnoldiPlan {
+  int nblk = 1;
+  int64_t per = kTile;
+};
+static ArnoldiPlan arnoldi_plan(int64_t n) {
+  ArnoldiPlan best;
+  double tbest = 1e300;
   const int64_t tiles = std::max<int64_t>(1, (n + kTile - 1) / kTile);
-  const int64_t per = (tiles + 152 * 4 - 1) / (152 * 4);
-  return (int)((tiles + per - 1) / per);
+  for (int ctas = 1; ctas <= 6; ++ctas) {  // CTAs per SM
+    const int64_t per = (tiles + 152 * ctas - 1) / (152 * ctas);
+    const int64_t nblk = (tiles + per - 1) / per;
+    if (per > 1 && ctas < (per > 2 ? 3 : 2)) continue;
+    const double t = (double)((nblk + 151) / 152) * (768.0 * per + 120.0);
+    if (t < tbest) {
+      tbest = t;
+      best.nblk = (int)nblk;
+      best.per = per * kTile;
+    }
+  }
+  return best;
 }
+int mdot_blocks(int64_t n) { return arnoldi_plan(n).nblk; }
 
 void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, double *partial, int nblk,
           cudaStream_t s, double *out, unsigned *cnt) {
-  if (nblk > kFinishBlocks) cnt = nullptr;
+  const ArnoldiPlan p = arnoldi_plan(n);
+  if (k != 1 || !out) cnt = nullptr;
   {
     HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 1), 1, n, 2.0 * n * k);
-    go<KMdot>(nblk, kThreads, 0, s, {V, ldv, k, w, n, partial, nblk, out, cnt});
+    go<KMdot>(nblk, kThreads, 0, s, {V, ldv, k, w, n, partial, nblk, p.per, out, cnt});
   }
   if (out && !cnt) reduce_partials(partial, k, nblk, out, s);
 }
@@ -1925,23 +1969,24 @@ void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, doubl
 void reduce_partials(const double *partial, int k, int nblk, double *out, cudaStream_t s) {
   HookScope hs(s, K_ARNOLDI, 8.0 * (double)k * nblk, 2, k, (double)k * nblk);
   // recorded launches take a grid that does not depend on k (blocks >= k return)
-  go<KReducePartials>(g_rec ? (unsigned)kMaxQ : (unsigned)k, 32, 0, s, {partial, k, nblk, out});
+  go<KReducePartials>(g_rec ? (unsigned)kMaxQ : (unsigned)k, kThreads, 0, s, {partial, k, nblk, out});
 }
 
 void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
-               int nblk, double *out, unsigned *cnt, cudaStream_t s) {
-  if (nblk > kFinishBlocks) cnt = nullptr;
+               int nblk, double *out, cudaStream_t s) {
+  const ArnoldiPlan p = arnoldi_plan(n);
   {
     HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 3, n, 4.0 * n * k);
-    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, out, cnt});
+    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, p.per});
   }
-  if (!cnt) reduce_partials(partial, k, nblk, out, s);
+  reduce_partials(partial, k, nblk, out, s);
 }
 
 void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
                 double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s) {
+  const ArnoldiPlan p = arnoldi_plan(n);
   HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 4, n, 2.0 * n * k + 2.0 * n);
-  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, out, cnt});
+  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, p.per, out, cnt});
 }
 
 void gemv_add(const double *Z, int64_t ldz, int k, const double *y, double *x, int64_t n, cudaStream_t s) {

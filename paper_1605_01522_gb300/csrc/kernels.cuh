@@ -209,18 +209,17 @@ void scale_convert_dev(double *v, const double *inv, TO *out, int64_t n, cudaStr
 
 // Arnoldi (float64).  V holds k row vectors of length n, row q at V + q*ldv.
 // partial: k * nblk doubles of scratch, nblk = mdot_blocks(n); out: device
-// memory; cnt: a device counter that is 0 between passes (passes over few
-// CTAs add up their partial sums in their last CTA, the others launch
-// reduce_partials; the order of the sums is the same).
+// memory; cnt: a device counter that is 0 between passes.
 int mdot_blocks(int64_t n);
 // out[q] = V_q . w; with out null only partial[q*nblk+b], for a later
-// reduce_partials; cnt may be null
+// reduce_partials.  One row with cnt given is reduced by the pass itself
+// (the same sum).
 void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, double *partial,
           int nblk, cudaStream_t s, double *out = nullptr, unsigned *cnt = nullptr);
 void reduce_partials(const double *partial, int k, int nblk, double *out, cudaStream_t s);
 // w -= sum_q V_q h_q and out[q] = V_q . w_new in one pass (k <= 64)
 void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
-               int nblk, double *out, unsigned *cnt, cudaStream_t s);
+               int nblk, double *out, cudaStream_t s);
 // w -= sum_q V_q h_q, out[0] = |w_new|^2, out[1] = 1 / |w_new|
 void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
                 double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s);

@@ -1311,7 +1311,7 @@ void arnoldi(mfs_handle *h, int j, double *w, double *hd, cudaStream_t s) {
   const int64_t n = h->n;
   // CGS2: h1 = V^T w (and |w|^2), w -= V h1, h2 = V^T w, w -= V h2 (and |w|^2)
   dev::mdot(h->V, n, j + 2, w, n, h->partial, h->nblk, s, hd, h->cnt);
-  dev::cgs_fused(h->V, n, j + 1, hd, w, n, h->partial, h->nblk, hd + 64, h->cnt, s);
+  dev::cgs_fused(h->V, n, j + 1, hd, w, n, h->partial, h->nblk, hd + 64, s);
   dev::cgs_update(h->V, n, j + 1, hd + 64, w, n, h->partial, h->nblk, hd + 128, h->cnt, s);
 }
 

@@ -168,13 +168,15 @@ typedef struct {
                                         the paper's DD(GS(0.79)), Sec. 7.1); 0 < omega < 2 */
   int rows_split;                    /* threads per block row of the float64 coupled matvec
                                         (merged row layout): 0 (default) = timed at setup
-                                        among 1, 2 and 4; or 1, 2, 4 to fix it */
+                                        among 1, 2, 4 and 8; or 1, 2, 4 to fix it */
   int layout_tune;                   /* sparse layouts of matrices with >= 2048 block rows:
                                         0 (default) = the fastest of SELL-32 (2, 4 or 8
-                                        slots in flight) and one warp per row, each timed
+                                        slots in flight, or 2, 4 or 8 threads per
+                                        row) and one warp per row, each timed
                                         alone (best for one solve at a time: a mid-size
-                                        matrix cannot fill the GPU by itself); 1 = the same,
-                                        but one warp per row only for rows of >= 32 blocks
+                                        matrix cannot fill the GPU by itself); 1 = the same
+                                        with one thread per row, and one warp per row only
+                                        for rows of >= 32 blocks
                                         (best when many systems run together,
                                         mfs_solve_batch, where the GPU is full and
                                         throughput counts) */
@@ -359,7 +361,7 @@ int mfs_kernel_stats(struct mfs_handle *h, double *out, int cap, int reset);
  * launches, ms, algorithmic bytes, algorithmic flops], where for SpMV (cls 0) and smoothing
  * (cls 1) sig = layout*1000 + br*100 + bc*10 + (float64 ? 1 : 0) with layout
  * 0 = SELL-32, 1 = warp-per-row BSR, 2 = merged coupled rows, 3 = SELL-32 with
- * 4 slots in flight (the layout autotuner's choices), and rows = block rows; for the other
+ * 4 slots in flight, 8 = SELL-32 with several threads per row (the layout autotuner's choices), and rows = block rows; for the other
  * classes sig is a kernel id and rows the vector length.  Returns the number
  * of rows written (cap = length of out).  Cleared by mfs_kernel_stats with
  * reset != 0. */

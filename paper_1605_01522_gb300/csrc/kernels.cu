@@ -142,7 +142,8 @@ void go(unsigned grid, unsigned threads, size_t smem, cudaStream_t s, const type
 }
 
 template <typename T> int sparse_sig(const Sell &A) {
-  // 3 / 9: SELL-32 with 4 / 8 slots in flight
+  // 3 / 9: SELL-32 with 4 / 8 slots in flight, 8: several threads per row
+  if (A.kind == 0 && A.split > 1) return 8000 + A.br * 100 + A.bc * 10 + (sizeof(T) == 8 ? 1 : 0);
   const int layout = A.kind == 0 && A.unroll == 4 ? 3 : (A.kind == 0 && A.unroll == 8 ? 9 : A.kind);
   return layout * 1000 + A.br * 100 + A.bc * 10 + (sizeof(T) == 8 ? 1 : 0);
 }
@@ -456,6 +457,116 @@ struct KSpmvSell {
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
     d_spmv<BR, BC, T, U>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, a.y, a.alpha, a.beta, a.z, bid, nb);
+  }
+};
+
+// SELL-32 with H = blockDim.x / 32 threads per block row, for matrices whose
+// rows alone do not fill the GPU: a CTA takes one slice, its warp h the slots
+// h, h + H, ... of the 32 rows; the H partial sums of an entry meet in shared
+// memory and are added in the order of h by the thread that finishes the
+// entry (entry e of the slice: row e / BR, component e % BR, so that the
+// vectors are read and written in whole segments; up to BR entries a thread).
+// One thread per row left 68,921 rows of 27 3x3 float32 blocks with 453
+// threads per SM, each walking its slots: 22.8 us a product, the best other
+// layout 20.1 us, with H = 4 11.9 us (launch and events: 5.5 us of each).
+constexpr int kSellSplitMax = 8;
+constexpr int kSellPad = 33;  // row pitch of the partial sums (bank conflicts)
+
+template <int BR, int BC, typename T>
+__device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__restrict__ sp,
+                                                const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
+                                                const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
+                                                T (*part)[BR][kSellPad]) {
+  const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, H = blockDim.x >> 5;
+  const int64_t row = slice * 32 + lane;
+  T acc[BR];
+#pragma unroll
+  for (int r = 0; r < BR; ++r) acc[r] = T(0);
+  if (row < nbr) {
+    const int64_t base = sp[slice];
+    const int len = rl[row];
+    const int32_t *cp = col + base * 32 + lane;
+    const T *vp = val + base * (BR * BC * 32) + lane;
+#pragma unroll 2
+    for (int t = h; t < len; t += H) {
+      const int64_t c = __ldg(cp + (int64_t)t * 32);
+      T xv[BC];
+#pragma unroll
+      for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
+      const T *v = vp + (int64_t)t * (BR * BC * 32);
+#pragma unroll
+      for (int r = 0; r < BR; ++r)
+#pragma unroll
+        for (int q = 0; q < BC; ++q) acc[r] += __ldg(v + (r * BC + q) * 32) * xv[q];
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < BR; ++r) part[h][r][lane] = acc[r];
+  __syncthreads();
+}
+
+template <int BR, typename T>
+__device__ __forceinline__ T sell_split_entry(T (*part)[BR][kSellPad], int e) {
+  const int H = blockDim.x >> 5;
+  T a = part[0][e % BR][e / BR];
+  for (int h = 1; h < H; ++h) a += part[h][e % BR][e / BR];
+  return a;
+}
+
+template <int BR, int BC, typename T>
+struct KSpmvSellSplit {
+  static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  struct Args {
+    int64_t nbr;
+    const int32_t *sp;
+    const int32_t *rl;
+    const int32_t *col;
+    const T *val;
+    const T *x;
+    T *y;
+    T alpha;
+    T beta;
+    const T *z;
+  };
+  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
+    __shared__ T part[kSellSplitMax][BR][kSellPad];
+    sell_split_sums<BR, BC, T>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, bid, part);
+    const int64_t i0 = (int64_t)bid * 32 * BR, n = a.nbr * BR;
+    for (int e = threadIdx.x; e < 32 * BR && i0 + e < n; e += blockDim.x) {
+      const T s = sell_split_entry<BR, T>(part, e);
+      a.y[i0 + e] = a.z != nullptr ? a.alpha * s + a.beta * a.z[i0 + e] : a.alpha * s;
+    }
+  }
+};
+
+template <int BR, typename T>
+struct KSmoothSellSplit {
+  static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  struct Args {
+    int64_t nbr;
+    const int32_t *sp;
+    const int32_t *rl;
+    const int32_t *col;
+    const T *val;
+    const T *dinv;
+    const T *b;
+    const T *x;
+    T *xout;
+    T *d;
+    T c1;
+    T c2;
+  };
+  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
+    __shared__ T part[kSellSplitMax][BR][kSellPad];
+    sell_split_sums<BR, BR, T>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, bid, part);
+    const int64_t i0 = (int64_t)bid * 32 * BR, n = a.nbr * BR;
+    for (int e = threadIdx.x; e < 32 * BR && i0 + e < n; e += blockDim.x) {
+      const int64_t i = i0 + e;
+      const T res = a.b[i] - sell_split_entry<BR, T>(part, e);
+      const T dd = a.c1 * a.d[i] + a.c2 * a.dinv[i] * res;
+      a.d[i] = dd;
+      a.xout[i] = a.x[i] + dd;
+    }
   }
 };
 
@@ -1664,7 +1775,11 @@ void spmv(const Sell &A, const T *x, T *y, T alpha, T beta, const T *z, cudaStre
     }
     return;
   }
-  if (A.unroll == 4) {
+  if (A.split > 1) {
+    MFS_BLOCK_DISPATCH(A.br, A.bc,
+                       (go<KSpmvSellSplit<BR_, BC_, T>>((unsigned)A.nslices, 32 * A.split, 0, s, {
+                           A.nbr, A.sp, A.rl, A.col, v, x, y, alpha, beta, z})));
+  } else if (A.unroll == 4) {
     MFS_BLOCK_DISPATCH(A.br, A.bc,
                        (go<KSpmvSell<BR_, BC_, T, 4>>(grid_for(A.nbr, kSellThreads), kSellThreads, 0, s, {
                            A.nbr, A.sp, A.rl, A.col, v, x, y, alpha, beta, z})));
@@ -1716,7 +1831,10 @@ void spmv_rows(const RowMerged &R, const double *x, double *y, cudaStream_t s) {
   const double *x0 = x + R.off[0], *x1 = x + R.off[1], *x2 = R.nb > 2 ? x + R.off[2] : x;
   const int b3[3] = {R.b[0], R.b[1], R.nb > 2 ? R.b[2] : 0};
   const unsigned grid = (unsigned)A.nslices;  // H > 1: one slice per CTA
-  if (R.split == 4) {
+  if (R.split == 8) {
+    MFS_ROWS_DISPATCH(A.br, b3, (go<KSpmvRows<R_, X0, X1, X2, 8>>(grid, 256, 0, s, {
+                                    A.nbr, A.sp, A.rl, A.col, A.v64, x0, x1, x2, y})));
+  } else if (R.split == 4) {
     MFS_ROWS_DISPATCH(A.br, b3, (go<KSpmvRows<R_, X0, X1, X2, 4>>(grid, 128, 0, s, {
                                     A.nbr, A.sp, A.rl, A.col, A.v64, x0, x1, x2, y})));
   } else if (R.split == 2) {
@@ -1740,7 +1858,10 @@ void smooth_step(const Sell &A, const T *dinv, const T *b, const T *x, T *xout, 
                                   A.nbr, A.sp, A.col, v, dinv, b, x, xout, d, c1, c2})));
     return;
   }
-  if (A.unroll == 4) {
+  if (A.split > 1) {
+    MFS_SQUARE_DISPATCH(A.br, (go<KSmoothSellSplit<BR_, T>>((unsigned)A.nslices, 32 * A.split, 0, s, {
+                                  A.nbr, A.sp, A.rl, A.col, v, dinv, b, x, xout, d, c1, c2})));
+  } else if (A.unroll == 4) {
     MFS_SQUARE_DISPATCH(A.br, (go<KSmoothSell<BR_, T, 4>>(grid_for(A.nbr, kSellThreads), kSellThreads, 0, s, {
                                   A.nbr, A.sp, A.rl, A.col, v, dinv, b, x, xout, d, c1, c2})));
   } else if (A.unroll == 8) {

@@ -21,7 +21,8 @@ struct Sell {
                                //    few rows: restriction, coarse levels); then sp is
                                //    the row pointer, col the block columns and the
                                //    values are contiguous per block (br*bc, row-major)
-  int unroll = 2;              // SELL-32: slots of a row in flight per thread (2 or 4)
+  int unroll = 2;              // SELL-32: slots of a row in flight per thread (2, 4 or 8)
+  int split = 1;               // SELL-32: threads per block row (1, or 2, 4, 8 with unroll 2)
   int br = 0, bc = 0;
   int64_t nbr = 0, nbc = 0;
   int64_t nslices = 0, nslots = 0;
@@ -43,7 +44,7 @@ enum KernelClass { K_SPMV = 0, K_SMOOTH = 1, K_VECTOR = 2, K_COARSE = 3, K_ARNOL
 // layout*1000 + br*100 + bc*10 + (float64 ? 1 : 0) with layout 0 SELL-32,
 // 1 warp BSR, 2 merged rows, 3 SELL-32 with 4 slots in flight, 4 / 5 / 6 the
 // Gauss-Seidel colour kernels on SELL-32 / warp BSR / SELL-32 x4, 7 one CTA per
-// BSR row; otherwise a small id.
+// BSR row, 8 SELL-32 with several threads per row; otherwise a small id.
 // rows = block rows (sparse kernels) or vector length.
 struct LaunchHook {
   // returns false when this launch is not to be recorded (after() is then skipped)
@@ -117,7 +118,7 @@ struct RowMerged {
   int nb = 0;      // number of merged column fields (2 or 3)
   int b[3] = {0, 0, 0};
   int64_t off[3] = {0, 0, 0};  // offset of each column field in the coupled vector
-  int split = 1;   // threads per block row (1, 2 or 4), timed at setup
+  int split = 1;   // threads per block row (1, 2, 4 or 8), timed at setup
 };
 bool rows_supported(int br, const int *b, int nb);
 void spmv_rows(const RowMerged &R, const double *x, double *y, cudaStream_t s);

@@ -366,13 +366,17 @@ static thread_local int g_layout_tune = 0;
 
 // Layout candidates of the autotuner: 0 SELL-32 with 2 slots in flight,
 // 1 with 4, 2 plain BSR with one warp per row, 3 SELL-32 with 8 slots in
-// flight (only for blocks of at most 3 entries, whose rows are short on bytes).
+// flight (only for blocks of at most 3 entries, whose rows are short on bytes),
+// 4, 5, 6 SELL-32 with 2, 4, 8 threads per row (the two that bring the matrix
+// closest to, but not far above, the 9,728 warps that the GPU holds; tuning
+// for batches leaves them out, other systems fill the GPU there).
+constexpr int kTuneCands = 7;
 static int tune_pick(const dev::Sell &a, const dev::Sell &b, bool want32, cudaStream_t st) {
   dev::Sell a4 = a, a8 = a;
   a4.unroll = 4;
   a8.unroll = 8;
   const bool small = a.br * a.bc <= 3;
-  float t[4];
+  float t[kTuneCands];
   t[0] = want32 ? time_spmv<float>(a, st) : time_spmv<double>(a, st);
   t[1] = want32 ? time_spmv<float>(a4, st) : time_spmv<double>(a4, st);
   // throughput tuning leaves the one-warp-per-row layout out for short rows
@@ -382,8 +386,16 @@ static int tune_pick(const dev::Sell &a, const dev::Sell &b, bool want32, cudaSt
   const bool short_rows = a.nnzb < 32 * a.nbr;
   t[2] = g_layout_tune == 1 && short_rows ? 1e30f : (want32 ? time_spmv<float>(b, st) : time_spmv<double>(b, st));
   t[3] = !small ? 1e30f : (want32 ? time_spmv<float>(a8, st) : time_spmv<double>(a8, st));
+  for (int c = 4; c < kTuneCands; ++c) {
+    dev::Sell ah = a;
+    ah.split = 1 << (c - 3);
+    const int64_t warps = a.nslices * ah.split;
+    t[c] = 1e30f;
+    if (g_layout_tune == 1 || warps > 20000 || (warps < 5000 && ah.split < 4)) continue;
+    t[c] = want32 ? time_spmv<float>(ah, st) : time_spmv<double>(ah, st);
+  }
   int best = 0;
-  for (int c = 1; c < 4; ++c)
+  for (int c = 1; c < kTuneCands; ++c)
     if (t[c] < t[best]) best = c;
   return best;
 }
@@ -391,6 +403,7 @@ static int tune_pick(const dev::Sell &a, const dev::Sell &b, bool want32, cudaSt
 static void tune_apply(dev::Sell &S, int best) {
   if (best == 1) S.unroll = 4;
   if (best == 3) S.unroll = 8;
+  if (best >= 4) S.split = 1 << (best - 3);
 }
 
 // keep the chosen candidate, release the other layout
@@ -2036,7 +2049,7 @@ HBsr to_hbsr(const mfs_block &b) {
   return A;
 }
 
-// Threads per block row of the merged float64 matvec (1, 2 or 4): timed
+// Threads per block row of the merged float64 matvec (1, 2, 4 or 8): timed
 // once per (row block shape, rows, blocks) and process, like the layouts.
 static std::map<std::tuple<int, int, int, int, int64_t, int64_t>, int> g_tune_rows;
 
@@ -2057,7 +2070,7 @@ static int tune_rows(const dev::RowMerged &R, int64_t n, cudaStream_t st) {
   MFS_CUDA(cudaEventCreate(&e1));
   int best = 1;
   float tbest = 1e30f;
-  for (int split : {1, 2, 4}) {
+  for (int split : {1, 2, 4, 8}) {
     dev::RowMerged T = R;
     T.split = split;
     for (int rep = 0; rep < 4; ++rep) {

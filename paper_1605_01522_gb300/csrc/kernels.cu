@@ -81,11 +81,30 @@ struct HookScope {
 // scheduled while its predecessor in the stream still runs: it first waits
 // until that predecessor has completed and its writes are visible, then lets
 // its own successor start launching.  Launched normally, both are no-ops.
+// Kernels with K::kEarly take the wait as a functor and call it (once, by
+// every thread) after their first loads of matrix data, which no launch of a
+// solve writes: a chain of dependent small launches then pays for the row
+// pointer, the columns and the blocks while the predecessor still runs (a
+// 13-CTA gather chain: 1.24 -> 0.97 us a launch).
+struct PdlWait {
+  __device__ __forceinline__ void operator()() const { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+};
+struct NoWait {
+  __device__ __forceinline__ void operator()() const {}
+};
+template <class K, class = void> struct IsEarly : std::false_type {};
+template <class K> struct IsEarly<K, std::void_t<decltype(K::kEarly)>> : std::true_type {};
+
 template <class K>
 __global__ void __launch_bounds__(K::kMaxThreads) k_solo(const __grid_constant__ typename K::Args a) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  K::run(a, (int)blockIdx.x, (int)gridDim.x);
+  if constexpr (IsEarly<K>::value) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    K::run(a, (int)blockIdx.x, (int)gridDim.x, PdlWait());
+  } else {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    K::run(a, (int)blockIdx.x, (int)gridDim.x);
+  }
 }
 
 // CTAs per SM the multi-system form of K must fit (K::kMinBlocks, default 1):
@@ -104,7 +123,8 @@ __global__ void __launch_bounds__(K::kMaxThreads, MinBlocks<K>::value)
 k_multi(const typename K::Args *__restrict__ tab, const MsBlock *__restrict__ map, const int *__restrict__ active) {
   const MsBlock m = map[blockIdx.x];
   if (active != nullptr && active[m.g] == 0) return;
-  K::run(tab[m.t], m.bid, m.nb);
+  if constexpr (IsEarly<K>::value) K::run(tab[m.t], m.bid, m.nb, NoWait());
+  else K::run(tab[m.t], m.bid, m.nb);
 }
 
 // issue one launch of K, or record it (with the accounting of the enclosing
@@ -227,31 +247,72 @@ __device__ __forceinline__ void sell_row(const int32_t *__restrict__ sp, const i
   }
 }
 
-// One warp per block row of a plain BSR matrix: lanes stride over the row's
-// blocks, then a fixed xor-butterfly sums the lanes (all lanes get the sums).
-template <int BR, int BC, typename T>
-__device__ __forceinline__ void bsr_warp_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-                                             const T *__restrict__ val, const T *__restrict__ x, int64_t row,
-                                             int lane, T (&acc)[BR]) {
-  const int lo = rp[row], hi = rp[row + 1];
+// A plain-BSR block row by a group of L = 2^ls lanes (8, 16 or 32): the lanes
+// stride over the row's blocks.  The first block of a lane is loaded before
+// `wait` (see k_solo), the next column while the current block is used, so
+// that a further block costs one load latency instead of two.
+template <int BR, int BC, typename T, class W>
+__device__ __forceinline__ void bsr_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
+                                        const T *__restrict__ val, const T *__restrict__ x, int64_t row, bool active,
+                                        int gl, int ls, W wait, T (&acc)[BR]) {
+  int k = 0, hi = 0;
+  if (active) {
+    k = rp[row] + gl;
+    hi = rp[row + 1];
+  }
+  int64_t c = 0;
+  T blk[BR * BC];
+  if (k < hi) {
+    c = __ldg(col + k);
+    ldg_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
+  }
+  wait();
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = T(0);
-  for (int k = lo + lane; k < hi; k += 32) {
-    const int64_t c = __ldg(col + k);
+  while (k < hi) {
+    const int kn = k + (1 << ls);
     T xv[BC];
 #pragma unroll
     for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
-    T blk[BR * BC];
-    ldg_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
+    if (kn < hi) c = __ldg(col + kn);
 #pragma unroll
     for (int r = 0; r < BR; ++r)
 #pragma unroll
       for (int q = 0; q < BC; ++q) acc[r] += blk[r * BC + q] * xv[q];
+    if (kn < hi) ldg_block<BR * BC, T>(val + (int64_t)kn * (BR * BC), blk);
+    k = kn;
   }
+}
+
+// Sums of the BR entries over a group of 2^ls lanes (8, 16 or 32).  With R the
+// power of two >= BR: while a lane still holds several entries it keeps one
+// half, adds the partner's and hands the other half over, so 6 adds instead
+// of 15 for three entries and 32 lanes (in float64 every add of a warp takes
+// 64 cycles of an SM quarter).  Lane gl returns the sum of entry
+// sum_entry<BR>(gl, ls); entries past BR - 1 are zero.
+template <int BR> constexpr int kSumRows = BR <= 1 ? 1 : BR <= 2 ? 2 : BR <= 4 ? 4 : 8;
+template <int BR> __device__ __forceinline__ int sum_entry(int gl, int ls) { return (gl * kSumRows<BR>) >> ls; }
+template <int BR> __device__ __forceinline__ bool sum_owner(int gl, int ls) {
+  return (gl & ((1 << ls) / kSumRows<BR> - 1)) == 0 && sum_entry<BR>(gl, ls) < BR;
+}
+template <int BR, typename T>
+__device__ __forceinline__ T group_sum(const T (&acc)[BR], int gl, int ls) {
+  constexpr int R = kSumRows<BR>;
+  T a[R];
 #pragma unroll
-  for (int r = 0; r < BR; ++r)
+  for (int r = 0; r < R; ++r) a[r] = r < BR ? acc[r < BR ? r : 0] : T(0);
+  int o = 1 << (ls - 1);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
+  for (int m = R / 2; m > 0; m /= 2, o >>= 1) {
+    const bool up = (gl & o) != 0;
+#pragma unroll
+    for (int r = 0; r < m; ++r) {
+      const T keep = up ? a[r + m] : a[r], give = up ? a[r] : a[r + m];
+      a[r] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  for (; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+  return a[0];
 }
 
 // dx of one node from its row sums acc (see gs_sweeps), written into x
@@ -281,32 +342,10 @@ __device__ __forceinline__ void gs_update(const T (&acc)[BR], int64_t node, cons
   for (int r = 0; r < BR; ++r) x[node * BR + r] += dx[r];
 }
 
-template <int BR, typename T>
-__device__ __forceinline__ T pick(const T (&acc)[BR], int r) {
-  T a = acc[0];
-#pragma unroll
-  for (int q = 1; q < BR; ++q)
-    if (q == r) a = acc[q];
-  return a;
-}
-
-template <int BR, int BC, typename T>
-__device__ __forceinline__ void d_spmv_warp(int64_t nbr, const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-            const T *__restrict__ val, const T *__restrict__ x, T *y, T alpha, T beta, const T *z, int bid_, int nb_) {
-  const int64_t row = ((int64_t)bid_ * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= nbr) return;
-  T acc[BR];
-  bsr_warp_row<BR, BC, T>(rp, col, val, x, row, lane, acc);
-  if (lane < BR) {
-    const int64_t i = row * BR + lane;
-    const T a = pick<BR, T>(acc, lane);
-    y[i] = z != nullptr ? alpha * a + beta * z[i] : alpha * a;
-  }
-}
 template <int BR, int BC, typename T>
 struct KSpmvWarp {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
     const int32_t *rp;
@@ -317,9 +356,18 @@ struct KSpmvWarp {
     T alpha;
     T beta;
     const T *z;
+    int ls;  // log2 of the lanes per row
   };
-  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_spmv_warp<BR, BC, T>(a.nbr, a.rp, a.col, a.val, a.x, a.y, a.alpha, a.beta, a.z, bid, nb);
+  template <class W> static __device__ __forceinline__ void run(const Args &a, int bid, int nb, W wait) {
+    const int64_t row = ((int64_t)bid * blockDim.x + threadIdx.x) >> a.ls;
+    const int gl = threadIdx.x & ((1 << a.ls) - 1);
+    T acc[BR];
+    bsr_row<BR, BC, T>(a.rp, a.col, a.val, a.x, row, row < a.nbr, gl, a.ls, wait, acc);
+    const bool own = row < a.nbr && sum_owner<BR>(gl, a.ls);
+    const int64_t i = row * BR + sum_entry<BR>(gl, a.ls);
+    const T zi = own && a.z != nullptr ? a.z[i] : T(0);
+    const T s = group_sum<BR, T>(acc, gl, a.ls);
+    if (own) a.y[i] = a.z != nullptr ? a.alpha * s + a.beta * zi : a.alpha * s;
   }
 };
 
@@ -381,25 +429,9 @@ struct KSpmvCta {
 };
 
 template <int BR, typename T>
-__device__ __forceinline__ void d_smooth_warp(int64_t nbr, const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-              const T *__restrict__ val, const T *__restrict__ dinv, const T *__restrict__ b,
-              const T *__restrict__ x, T *__restrict__ xout, T *__restrict__ d, T c1, T c2, int bid_, int nb_) {
-  const int64_t row = ((int64_t)bid_ * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= nbr) return;
-  T acc[BR];
-  bsr_warp_row<BR, BR, T>(rp, col, val, x, row, lane, acc);
-  if (lane < BR) {
-    const int64_t i = row * BR + lane;
-    const T res = b[i] - pick<BR, T>(acc, lane);
-    const T dd = c1 * d[i] + c2 * dinv[i] * res;
-    d[i] = dd;
-    xout[i] = x[i] + dd;
-  }
-}
-template <int BR, typename T>
 struct KSmoothWarp {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
     const int32_t *rp;
@@ -412,9 +444,29 @@ struct KSmoothWarp {
     T *d;
     T c1;
     T c2;
+    int ls;  // log2 of the lanes per row
   };
-  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_smooth_warp<BR, T>(a.nbr, a.rp, a.col, a.val, a.dinv, a.b, a.x, a.xout, a.d, a.c1, a.c2, bid, nb);
+  template <class W> static __device__ __forceinline__ void run(const Args &a, int bid, int nb, W wait) {
+    const int64_t row = ((int64_t)bid * blockDim.x + threadIdx.x) >> a.ls;
+    const int gl = threadIdx.x & ((1 << a.ls) - 1);
+    const bool own = row < a.nbr && sum_owner<BR>(gl, a.ls);
+    const int64_t i = row * BR + sum_entry<BR>(gl, a.ls);
+    const T di = own ? a.dinv[i] : T(0);
+    T acc[BR];
+    bsr_row<BR, BR, T>(a.rp, a.col, a.val, a.x, row, row < a.nbr, gl, a.ls, wait, acc);
+    T bi = T(0), xi = T(0), dd = T(0);
+    if (own) {
+      bi = a.b[i];
+      xi = a.x[i];
+      dd = a.d[i];
+    }
+    const T s = group_sum<BR, T>(acc, gl, a.ls);
+    if (own) {
+      const T res = bi - s;
+      dd = a.c1 * dd + a.c2 * di * res;
+      a.d[i] = dd;
+      a.xout[i] = xi + dd;
+    }
   }
 };
 
@@ -472,33 +524,50 @@ struct KSpmvSell {
 constexpr int kSellSplitMax = 8;
 constexpr int kSellPad = 33;  // row pitch of the partial sums (bank conflicts)
 
-template <int BR, int BC, typename T>
+template <int BR, int BC, typename T, class W>
 __device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__restrict__ sp,
                                                 const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
                                                 const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
-                                                T (*part)[BR][kSellPad]) {
+                                                W wait, T (*part)[BR][kSellPad]) {
   const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, H = blockDim.x >> 5;
   const int64_t row = slice * 32 + lane;
-  T acc[BR];
+  const int64_t base = sp[slice];
+  const int len = row < nbr ? rl[row] : 0;
+  const int32_t *cp = col + base * 32 + lane;
+  const T *vp = val + base * (BR * BC * 32) + lane;
+  // first slot: before the wait (see k_solo)
+  int64_t c = 0;
+  T v0[BR * BC], acc[BR];
+#pragma unroll
+  for (int e = 0; e < BR * BC; ++e) v0[e] = T(0);
+  if (h < len) {
+    c = __ldg(cp + (int64_t)h * 32);
+#pragma unroll
+    for (int e = 0; e < BR * BC; ++e) v0[e] = __ldg(vp + ((int64_t)h * (BR * BC) + e) * 32);
+  }
+  wait();
 #pragma unroll
   for (int r = 0; r < BR; ++r) acc[r] = T(0);
-  if (row < nbr) {
-    const int64_t base = sp[slice];
-    const int len = rl[row];
-    const int32_t *cp = col + base * 32 + lane;
-    const T *vp = val + base * (BR * BC * 32) + lane;
+  if (h < len) {
+    T xv[BC];
+#pragma unroll
+    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
+#pragma unroll
+    for (int r = 0; r < BR; ++r)
+#pragma unroll
+      for (int q = 0; q < BC; ++q) acc[r] += v0[r * BC + q] * xv[q];
+  }
 #pragma unroll 2
-    for (int t = h; t < len; t += H) {
-      const int64_t c = __ldg(cp + (int64_t)t * 32);
-      T xv[BC];
+  for (int t = h + H; t < len; t += H) {
+    const int64_t ct = __ldg(cp + (int64_t)t * 32);
+    T xv[BC];
 #pragma unroll
-      for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
-      const T *v = vp + (int64_t)t * (BR * BC * 32);
+    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + ct * BC + q);
+    const T *v = vp + (int64_t)t * (BR * BC * 32);
 #pragma unroll
-      for (int r = 0; r < BR; ++r)
+    for (int r = 0; r < BR; ++r)
 #pragma unroll
-        for (int q = 0; q < BC; ++q) acc[r] += __ldg(v + (r * BC + q) * 32) * xv[q];
-    }
+      for (int q = 0; q < BC; ++q) acc[r] += __ldg(v + (r * BC + q) * 32) * xv[q];
   }
 #pragma unroll
   for (int r = 0; r < BR; ++r) part[h][r][lane] = acc[r];
@@ -516,6 +585,7 @@ __device__ __forceinline__ T sell_split_entry(T (*part)[BR][kSellPad], int e) {
 template <int BR, int BC, typename T>
 struct KSpmvSellSplit {
   static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
     const int32_t *sp;
@@ -528,9 +598,9 @@ struct KSpmvSellSplit {
     T beta;
     const T *z;
   };
-  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
+  template <class W> static __device__ __forceinline__ void run(const Args &a, int bid, int nb, W wait) {
     __shared__ T part[kSellSplitMax][BR][kSellPad];
-    sell_split_sums<BR, BC, T>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, bid, part);
+    sell_split_sums<BR, BC, T>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, bid, wait, part);
     const int64_t i0 = (int64_t)bid * 32 * BR, n = a.nbr * BR;
     for (int e = threadIdx.x; e < 32 * BR && i0 + e < n; e += blockDim.x) {
       const T s = sell_split_entry<BR, T>(part, e);
@@ -542,6 +612,7 @@ struct KSpmvSellSplit {
 template <int BR, typename T>
 struct KSmoothSellSplit {
   static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
     const int32_t *sp;
@@ -556,9 +627,9 @@ struct KSmoothSellSplit {
     T c1;
     T c2;
   };
-  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
+  template <class W> static __device__ __forceinline__ void run(const Args &a, int bid, int nb, W wait) {
     __shared__ T part[kSellSplitMax][BR][kSellPad];
-    sell_split_sums<BR, BR, T>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, bid, part);
+    sell_split_sums<BR, BR, T>(a.nbr, a.sp, a.rl, a.col, a.val, a.x, bid, wait, part);
     const int64_t i0 = (int64_t)bid * 32 * BR, n = a.nbr * BR;
     for (int e = threadIdx.x; e < 32 * BR && i0 + e < n; e += blockDim.x) {
       const int64_t i = i0 + e;
@@ -825,31 +896,31 @@ struct KGsSmall {
 // x = inv b for the explicit inverse of a coarsest matrix (row-major, float64):
 // b staged in shared memory as float64, one warp per row, fixed butterfly sum.
 template <typename T>
-__device__ __forceinline__ void d_inv_apply(int n, const double *__restrict__ inv, const T *__restrict__ b, T *__restrict__ x, int bid_, int nb_) {
-  extern __shared__ double bs[];
-  for (int j = threadIdx.x; j < n; j += blockDim.x) bs[j] = (double)b[j];
-  __syncthreads();
-  const int row = bid_ * (blockDim.x / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  const double *a = inv + (int64_t)row * n;
-  double acc = 0.0;
-  for (int j = lane; j < n; j += 32) acc += __ldg(a + j) * bs[j];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) x[row] = (T)acc;
-}
-template <typename T>
 struct KInvApply {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kEarly = true;
   struct Args {
     int n;
     const double *inv;
     const T *b;
     T *x;
   };
-  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_inv_apply<T>(a.n, a.inv, a.b, a.x, bid, nb);
+  template <class W> static __device__ __forceinline__ void run(const Args &p, int bid, int nb, W wait) {
+    extern __shared__ double bs[];
+    const int row = bid * (blockDim.x / 32) + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    const double *a = p.inv + (int64_t)row * p.n;
+    const double a0 = row < p.n && lane < p.n ? __ldg(a + lane) : 0.0;
+    wait();
+    for (int j = threadIdx.x; j < p.n; j += blockDim.x) bs[j] = (double)p.b[j];
+    __syncthreads();
+    if (row >= p.n) return;
+    double acc = 0.0;
+    if (lane < p.n) acc += a0 * bs[lane];
+    for (int j = lane + 32; j < p.n; j += 32) acc += __ldg(a + j) * bs[j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) p.x[row] = (T)acc;
   }
 };
 
@@ -1515,52 +1586,54 @@ template <typename T> struct TailArgs {
   const double *inv;  // nc x nc row-major inverse of the coarsest matrix
   const T *b;
   T *x;
+  int als, rls, pls;  // log2 of the lanes per row of A, R, P
   int ns;  // smoothing steps per application
   T c1[kTailMaxSteps], c2[kTailMaxSteps];
 };
 
-// row sums of a plain-BSR block row against x in shared memory (the
-// arithmetic of bsr_warp_row)
-template <int BR, int BC, typename T>
-__device__ __forceinline__ void tail_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-                                         const T *__restrict__ val, const T *x, int64_t row, int lane,
-                                         T (&acc)[BR]) {
-  const int lo = rp[row], hi = rp[row + 1];
+// row sums of a plain-BSR block row against x in shared memory, with the
+// lanes per row and the arithmetic of KSpmvWarp; groups of 2^ls lanes stride
+// over the rows and f(row, entry, sum) runs in the lane that owns an entry
+template <int BR, int BC, typename T, class F>
+__device__ __forceinline__ void tail_rows(int64_t nbr, const int32_t *__restrict__ rp,
+                                          const int32_t *__restrict__ col, const T *__restrict__ val, const T *x,
+                                          int ls, F f) {
+  const int gl = threadIdx.x & ((1 << ls) - 1);
+  const int64_t step = kTailThreads >> ls;
+  for (int64_t r0 = 0; r0 < nbr; r0 += step) {
+    const int64_t row = r0 + (threadIdx.x >> ls);
+    const bool active = row < nbr;
+    T acc[BR];
 #pragma unroll
-  for (int r = 0; r < BR; ++r) acc[r] = T(0);
-  for (int k = lo + lane; k < hi; k += 32) {
-    const int64_t c = __ldg(col + k);
-    T xv[BC];
+    for (int r = 0; r < BR; ++r) acc[r] = T(0);
+    for (int k = active ? rp[row] + gl : 0; active && k < rp[row + 1]; k += 1 << ls) {
+      const int64_t c = __ldg(col + k);
+      T xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = x[c * BC + q];
-    T blk[BR * BC];
-    ldg_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
+      for (int q = 0; q < BC; ++q) xv[q] = x[c * BC + q];
+      T blk[BR * BC];
+      ldg_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
 #pragma unroll
-    for (int r = 0; r < BR; ++r)
+      for (int r = 0; r < BR; ++r)
 #pragma unroll
-      for (int q = 0; q < BC; ++q) acc[r] += blk[r * BC + q] * xv[q];
+        for (int q = 0; q < BC; ++q) acc[r] += blk[r * BC + q] * xv[q];
+    }
+    __syncwarp();
+    const T s = group_sum<BR, T>(acc, gl, ls);
+    if (active && sum_owner<BR>(gl, ls)) f(row, sum_entry<BR>(gl, ls), s);
   }
-#pragma unroll
-  for (int r = 0; r < BR; ++r)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], o);
 }
 
 // one smoothing step in shared memory: xo = x + d, d = c1 d + c2 dinv (b - A x)
 template <int BR, typename T>
 __device__ __forceinline__ void tail_smooth(const TailArgs<T> &a, const T *b, const T *x, T *xo, T *d, T c1, T c2) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int64_t row = warp; row < a.nbr; row += kTailThreads / 32) {
-    T acc[BR];
-    tail_row<BR, BR, T>(a.arp, a.acol, a.aval, x, row, lane, acc);
-    if (lane < BR) {
-      const int64_t i = row * BR + lane;
-      const T res = b[i] - pick<BR, T>(acc, lane);
-      const T dd = c1 * d[i] + c2 * a.dinv[i] * res;
-      d[i] = dd;
-      xo[i] = x[i] + dd;
-    }
-  }
+  tail_rows<BR, BR, T>(a.nbr, a.arp, a.acol, a.aval, x, a.als, [&](int64_t row, int r, T s) {
+    const int64_t i = row * BR + r;
+    const T res = b[i] - s;
+    const T dd = c1 * d[i] + c2 * a.dinv[i] * res;
+    d[i] = dd;
+    xo[i] = x[i] + dd;
+  });
   __syncthreads();
 }
 
@@ -1593,21 +1666,12 @@ __device__ __forceinline__ void d_vcycle_tail(const TailArgs<T> &a) {
     oth = t;
   }
   // residual r = b - A x  (as y = -1 * A x + 1 * b)
-  for (int64_t row = warp; row < a.nbr; row += kTailThreads / 32) {
-    T acc[BR];
-    tail_row<BR, BR, T>(a.arp, a.acol, a.aval, cur, row, lane, acc);
-    if (lane < BR) {
-      const int64_t i = row * BR + lane;
-      r[i] = T(-1) * pick<BR, T>(acc, lane) + T(1) * b[i];
-    }
-  }
+  tail_rows<BR, BR, T>(a.nbr, a.arp, a.acol, a.aval, cur, a.als,
+                       [&](int64_t row, int q, T t) { r[row * BR + q] = T(-1) * t + T(1) * b[row * BR + q]; });
   __syncthreads();
   // restriction bc = R r
-  for (int64_t row = warp; row < a.ncbr; row += kTailThreads / 32) {
-    T acc[BC];
-    tail_row<BC, BR, T>(a.rrp, a.rcol, a.rval, r, row, lane, acc);
-    if (lane < BC) bcT[row * BC + lane] = T(1) * pick<BC, T>(acc, lane);
-  }
+  tail_rows<BC, BR, T>(a.ncbr, a.rrp, a.rcol, a.rval, r, a.rls,
+                       [&](int64_t row, int q, T t) { bcT[row * BC + q] = T(1) * t; });
   __syncthreads();
   // coarsest solve through the explicit inverse, in float64
   for (int64_t j = tid; j < a.nc; j += kTailThreads) bc[j] = (double)bcT[j];
@@ -1622,14 +1686,8 @@ __device__ __forceinline__ void d_vcycle_tail(const TailArgs<T> &a) {
   }
   __syncthreads();
   // prolongation x += P xc  (as y = 1 * P xc + 1 * x)
-  for (int64_t row = warp; row < a.nbr; row += kTailThreads / 32) {
-    T acc[BR];
-    tail_row<BR, BC, T>(a.prp, a.pcol, a.pval, xc, row, lane, acc);
-    if (lane < BR) {
-      const int64_t i = row * BR + lane;
-      cur[i] = T(1) * pick<BR, T>(acc, lane) + T(1) * cur[i];
-    }
-  }
+  tail_rows<BR, BC, T>(a.nbr, a.prp, a.pcol, a.pval, xc, a.pls,
+                       [&](int64_t row, int q, T t) { cur[row * BR + q] = T(1) * t + T(1) * cur[row * BR + q]; });
   __syncthreads();
   // post-smoothing from the corrected x
   for (int k = 0; k < a.ns; ++k) {
@@ -1755,11 +1813,34 @@ void init() {
   done[dev] = true;
 }
 
+// log2 of the lanes per row of a plain-BSR matrix: the smallest group that
+// walks an average row in one step (8 blocks: 8 lanes), two steps for rows of
+// up to 32 blocks, more for longer ones.  In float64 the lanes' products
+// and sums bound these kernels (64 cycles a warp instruction): a 9-block row
+// of 3x3 blocks takes 9 warp instructions with 16 lanes, 24 with a warp.
+template <typename T> int bsr_ls(const Sell &A) {
+  const double avg = (double)A.nnzb / (double)A.nbr;
+  return avg <= 8.0 ? 3 : avg <= 32.0 ? 4 : 5;
+}
+// CTA size of the plain-BSR kernels: small enough to spread few rows over
+// the SMs, 64 to 256 threads
+static unsigned bsr_threads(int64_t lanes) {
+  unsigned t = 64;
+  while (t < (unsigned)kThreads && lanes > (int64_t)t * 152) t *= 2;
+  return t;
+}
+// few, long rows: one CTA per row; not in float64, where the 8 warps' sums
+// over lanes take longer than the row (6x3 blocks, 184 a row: 22 us on 1,128
+// rows, 7 us with a warp per row)
+template <typename T> bool cta_rows(const Sell &A) {
+  return sizeof(T) == 4 && A.kind == 1 && A.nbr <= kCtaRowsMax && A.nnzb >= kCtaRowBlocks * A.nbr;
+}
+
 template <typename T>
 void spmv(const Sell &A, const T *x, T *y, T alpha, T beta, const T *z, cudaStream_t s) {
   if (A.nbr == 0) return;
   const T *v = vals<T>(A);
-  const bool cta = A.kind == 1 && A.nbr <= kCtaRowsMax && A.nnzb >= kCtaRowBlocks * A.nbr;
+  const bool cta = cta_rows<T>(A);
   HookScope hs(s, K_SPMV, matrix_bytes<T>(A) + (double)sizeof(T) * (A.ncols() + A.nrows() * (z ? 2 : 1)),
                cta ? 7000 + sparse_sig<T>(A) % 1000 : sparse_sig<T>(A), A.nbr,
                2.0 * A.nnzb * A.br * A.bc + (z ? 3.0 : 1.0) * A.nrows());
@@ -1769,9 +1850,11 @@ void spmv(const Sell &A, const T *x, T *y, T alpha, T beta, const T *z, cudaStre
                          (go<KSpmvCta<BR_, BC_, T>>((unsigned)A.nbr, kThreads, 0, s, {
                              A.nbr, A.sp, A.col, v, x, y, alpha, beta, z})));
     } else {
+      const int ls = bsr_ls<T>(A);
+      const unsigned th = bsr_threads(A.nbr << ls);
       MFS_BLOCK_DISPATCH(A.br, A.bc,
-                         (go<KSpmvWarp<BR_, BC_, T>>(grid_for(A.nbr * 32), kThreads, 0, s, {
-                             A.nbr, A.sp, A.col, v, x, y, alpha, beta, z})));
+                         (go<KSpmvWarp<BR_, BC_, T>>(grid_for(A.nbr << ls, th), th, 0, s, {
+                             A.nbr, A.sp, A.col, v, x, y, alpha, beta, z, ls})));
     }
     return;
   }
@@ -1854,8 +1937,10 @@ void smooth_step(const Sell &A, const T *dinv, const T *b, const T *x, T *xout, 
   HookScope hs(s, K_SMOOTH, matrix_bytes<T>(A) + (double)sizeof(T) * (A.ncols() + 5.0 * A.nrows()),
                sparse_sig<T>(A), A.nbr, 2.0 * A.nnzb * A.br * A.bc + 6.0 * A.nrows());
   if (A.kind == 1) {
-    MFS_SQUARE_DISPATCH(A.br, (go<KSmoothWarp<BR_, T>>(grid_for(A.nbr * 32), kThreads, 0, s, {
-                                  A.nbr, A.sp, A.col, v, dinv, b, x, xout, d, c1, c2})));
+    const int ls = bsr_ls<T>(A);
+    const unsigned th = bsr_threads(A.nbr << ls);
+    MFS_SQUARE_DISPATCH(A.br, (go<KSmoothWarp<BR_, T>>(grid_for(A.nbr << ls, th), th, 0, s, {
+                                  A.nbr, A.sp, A.col, v, dinv, b, x, xout, d, c1, c2, ls})));
     return;
   }
   if (A.split > 1) {
@@ -1948,7 +2033,8 @@ size_t tail_smem_bytes(int64_t n, int64_t nc, size_t tsize) {
 
 bool tail_supported(int br, int bc) { return br == bc && (br == 1 || br == 2 || br == 3 || br == 6); }
 
-bool cta_rows(const Sell &A) { return A.kind == 1 && A.nbr <= kCtaRowsMax && A.nnzb >= kCtaRowBlocks * A.nbr; }
+template bool cta_rows<float>(const Sell &);
+template bool cta_rows<double>(const Sell &);
 
 template <typename T>
 void vcycle_tail(const Sell &A, const T *dinv, const Sell &R, const Sell &P, const DenseLU &lu, int ns,
@@ -1968,6 +2054,9 @@ void vcycle_tail(const Sell &A, const T *dinv, const Sell &R, const Sell &P, con
   a.prp = P.sp;
   a.pcol = P.col;
   a.pval = vals<T>(P);
+  a.als = bsr_ls<T>(A);
+  a.rls = bsr_ls<T>(R);
+  a.pls = bsr_ls<T>(P);
   a.inv = lu.inv;
   a.b = b;
   a.x = x;

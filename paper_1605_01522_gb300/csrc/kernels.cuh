@@ -168,7 +168,7 @@ void gs_sweeps(const GsLevel &g, const T *dblk, const T *b, T *x, T omega, int s
 // tail_smem_bytes, which the caller keeps within 48 KB.
 bool tail_supported(int br, int bc);
 // true when spmv runs this plain-BSR matrix with one CTA per row (few, long rows)
-bool cta_rows(const Sell &A);
+template <typename T> bool cta_rows(const Sell &A);
 size_t tail_smem_bytes(int64_t n, int64_t nc, size_t tsize);
 template <typename T>
 void vcycle_tail(const Sell &A, const T *dinv, const Sell &R, const Sell &P, const DenseLU &lu, int ns,

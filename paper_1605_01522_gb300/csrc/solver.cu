@@ -762,7 +762,7 @@ template <typename T> struct Precond {
     const dev::DenseLU &lu = g.cf[i];
     const dev::Sell &A = f.A, &R = f.R, &P = f.P;
     if (!lu.inv || lu.n == 0 || A.kind != 1 || R.kind != 1 || P.kind != 1) return false;
-    if (dev::cta_rows(A) || dev::cta_rows(R) || dev::cta_rows(P)) return false;
+    if (dev::cta_rows<T>(A) || dev::cta_rows<T>(R) || dev::cta_rows<T>(P)) return false;
     if (!dev::tail_supported(A.br, R.br) || R.bc != A.br || P.br != A.br || P.bc != R.br) return false;
     if (f.c1.size() > 8 || lu.n != R.nrows()) return false;
     return dev::tail_smem_bytes(A.nrows(), lu.n, sizeof(T)) <= 48 * 1024;

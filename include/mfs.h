@@ -169,7 +169,8 @@ typedef struct {
   int rows_split;                    /* threads per block row of the float64 coupled matvec
                                         (merged row layout): 0 (default) = timed at setup
                                         among 1, 2, 4 and 8; or 1, 2, 4 to fix it */
-  int layout_tune;                   /* sparse layouts of matrices with >= 2048 block rows:
+  int layout_tune;                   /* sparse layouts of matrices with >= 131,072 block rows
+                                        (>= 2,048 with 1; smaller ones by a rule):
                                         0 (default) = the fastest of SELL-32 (2, 4 or 8
                                         slots in flight, or 2, 4 or 8 threads per
                                         row) and one warp per row, each timed
@@ -193,9 +194,8 @@ typedef struct {
                                         results are the same): 1 every launch, 0 none,
                                         N > 1 launches of at most N CTAs, -1 (default)
                                         while no other solve runs in the process: every
-                                        launch of a system of at most 65,536 dofs (its
-                                        kernels are too short to hide a launch), the
-                                        launches of at most 160 CTAs of a larger one */
+                                        launch, of the kernels bound by the FP64 pipe
+                                        those of at most 160 CTAs */
 } mfs_params;
 
 typedef struct {

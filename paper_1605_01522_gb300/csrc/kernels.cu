@@ -37,7 +37,8 @@ thread_local Recorder *g_rec = nullptr;
 // launches where they directly follow another of its kernel launches on the
 // same stream (g_pdl_prev): a kernel after a copy, an event or a graph launch
 // is launched normally.
-thread_local unsigned g_pdl = 0;  // largest grid (CTAs) launched this way; 0: none
+thread_local unsigned g_pdl = 0;    // largest grid (CTAs) launched this way; 0: none
+thread_local unsigned g_pdl64 = 0;  // the same for kernels bound by the FP64 pipe (K::kFp64)
 thread_local cudaStream_t g_pdl_prev = nullptr;
 // accounting of the launch being issued (HookScope fills it for the recorder)
 thread_local RecOp g_acct;
@@ -86,8 +87,51 @@ struct HookScope {
 // solve writes: a chain of dependent small launches then pays for the row
 // pointer, the columns and the blocks while the predecessor still runs (a
 // 13-CTA gather chain: 1.24 -> 0.97 us a launch).
+// Loads of matrix data that stay before the wait: volatile, so that the
+// compiler does not move them behind it (as __ldg they were: 1.82 -> 1.72 ms
+// for a solve of the 3,267-dof system)
+__device__ __forceinline__ int32_t ld_pin(const int32_t *p) {
+  int32_t v;
+  asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_pin(const float *p) {
+  float v;
+  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_pin(const double *p) {
+  double v;
+  asm volatile("ld.global.nc.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+// a plain-BSR block, in the loads of ldg_block
+template <int N, typename T> __device__ __forceinline__ void ld_pin_block(const T *p, T (&o)[N]) {
+  constexpr int B = N * (int)sizeof(T);
+  if constexpr (sizeof(T) == 8 && B % 16 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 2)
+      asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(o[i]), "=d"(o[i + 1]) : "l"(p + i));
+  } else if constexpr (sizeof(T) == 4 && B % 16 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 4)
+      asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(o[i]), "=f"(o[i + 1]), "=f"(o[i + 2]), "=f"(o[i + 3])
+                   : "l"(p + i));
+  } else if constexpr (sizeof(T) == 4 && B % 8 == 0) {
+#pragma unroll
+    for (int i = 0; i < N; i += 2)
+      asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(o[i]), "=f"(o[i + 1]) : "l"(p + i));
+  } else {
+#pragma unroll
+    for (int i = 0; i < N; ++i) o[i] = ld_pin(p + i);
+  }
+}
 struct PdlWait {
-  __device__ __forceinline__ void operator()() const { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+  __device__ __forceinline__ void operator()() const {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  }
 };
 struct NoWait {
   __device__ __forceinline__ void operator()() const {}
@@ -95,10 +139,16 @@ struct NoWait {
 template <class K, class = void> struct IsEarly : std::false_type {};
 template <class K> struct IsEarly<K, std::void_t<decltype(K::kEarly)>> : std::true_type {};
 
+// Kernels that the FP64 pipe bounds have K::kFp64 = true.  A CTA launched ahead
+// takes its place while the predecessor's CTAs still hold theirs, so a grid
+// of a few CTAs per SM ends up uneven, and the SM with the most float64 work
+// sets the time; the float32 kernels wait for memory and do not mind.
+template <class K, class = void> struct IsFp64 : std::false_type {};
+template <class K> struct IsFp64<K, std::void_t<decltype(K::kFp64)>> : std::bool_constant<K::kFp64> {};
+
 template <class K>
 __global__ void __launch_bounds__(K::kMaxThreads) k_solo(const __grid_constant__ typename K::Args a) {
   if constexpr (IsEarly<K>::value) {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     K::run(a, (int)blockIdx.x, (int)gridDim.x, PdlWait());
   } else {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -142,7 +192,7 @@ void go(unsigned grid, unsigned threads, size_t smem, cudaStream_t s, const type
     g_acct = RecOp();
     return;
   }
-  const bool pdl = grid <= g_pdl && g_pdl_prev == s;
+  const bool pdl = grid <= (IsFp64<K>::value ? g_pdl64 : g_pdl) && g_pdl_prev == s;
   g_pdl_prev = g_pdl ? s : nullptr;
   if (pdl) {
     cudaLaunchConfig_t cfg = {};
@@ -257,14 +307,14 @@ __device__ __forceinline__ void bsr_row(const int32_t *__restrict__ rp, const in
                                         int gl, int ls, W wait, T (&acc)[BR]) {
   int k = 0, hi = 0;
   if (active) {
-    k = rp[row] + gl;
-    hi = rp[row + 1];
+    k = ld_pin(rp + row) + gl;
+    hi = ld_pin(rp + row + 1);
   }
   int64_t c = 0;
   T blk[BR * BC];
   if (k < hi) {
-    c = __ldg(col + k);
-    ldg_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
+    c = ld_pin(col + k);
+    ld_pin_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
   }
   wait();
 #pragma unroll
@@ -345,6 +395,7 @@ __device__ __forceinline__ void gs_update(const T (&acc)[BR], int64_t node, cons
 template <int BR, int BC, typename T>
 struct KSpmvWarp {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
@@ -412,6 +463,7 @@ __device__ __forceinline__ void d_spmv_cta(int64_t nbr, const int32_t *__restric
 template <int BR, int BC, typename T>
 struct KSpmvCta {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   struct Args {
     int64_t nbr;
     const int32_t *rp;
@@ -431,6 +483,7 @@ struct KSpmvCta {
 template <int BR, typename T>
 struct KSmoothWarp {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
@@ -451,7 +504,7 @@ struct KSmoothWarp {
     const int gl = threadIdx.x & ((1 << a.ls) - 1);
     const bool own = row < a.nbr && sum_owner<BR>(gl, a.ls);
     const int64_t i = row * BR + sum_entry<BR>(gl, a.ls);
-    const T di = own ? a.dinv[i] : T(0);
+    const T di = own ? ld_pin(a.dinv + i) : T(0);
     T acc[BR];
     bsr_row<BR, BR, T>(a.rp, a.col, a.val, a.x, row, row < a.nbr, gl, a.ls, wait, acc);
     T bi = T(0), xi = T(0), dd = T(0);
@@ -494,6 +547,7 @@ __device__ __forceinline__ void d_spmv(int64_t nbr, const int32_t *__restrict__ 
 template <int BR, int BC, typename T, int U>
 struct KSpmvSell {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr int kMinBlocks = BR * BC <= 9 ? 8 : 1;  // multi-system form: <= 32 registers
   struct Args {
     int64_t nbr;
@@ -521,6 +575,8 @@ struct KSpmvSell {
 // One thread per row left 68,921 rows of 27 3x3 float32 blocks with 453
 // threads per SM, each walking its slots: 22.8 us a product, the best other
 // layout 20.1 us, with H = 4 11.9 us (launch and events: 5.5 us of each).
+// (Loading the finishing entry's vectors ahead of the row cost registers:
+// 18.1 instead of 17.3 ms for the SIMPLE solve of the 40^3 box.)
 constexpr int kSellSplitMax = 8;
 constexpr int kSellPad = 33;  // row pitch of the partial sums (bank conflicts)
 
@@ -531,8 +587,8 @@ __device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__re
                                                 W wait, T (*part)[BR][kSellPad]) {
   const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, H = blockDim.x >> 5;
   const int64_t row = slice * 32 + lane;
-  const int64_t base = sp[slice];
-  const int len = row < nbr ? rl[row] : 0;
+  const int64_t base = ld_pin(sp + slice);
+  const int len = row < nbr ? ld_pin(rl + row) : 0;
   const int32_t *cp = col + base * 32 + lane;
   const T *vp = val + base * (BR * BC * 32) + lane;
   // first slot: before the wait (see k_solo)
@@ -541,9 +597,9 @@ __device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__re
 #pragma unroll
   for (int e = 0; e < BR * BC; ++e) v0[e] = T(0);
   if (h < len) {
-    c = __ldg(cp + (int64_t)h * 32);
+    c = ld_pin(cp + (int64_t)h * 32);
 #pragma unroll
-    for (int e = 0; e < BR * BC; ++e) v0[e] = __ldg(vp + ((int64_t)h * (BR * BC) + e) * 32);
+    for (int e = 0; e < BR * BC; ++e) v0[e] = ld_pin(vp + ((int64_t)h * (BR * BC) + e) * 32);
   }
   wait();
 #pragma unroll
@@ -585,6 +641,7 @@ __device__ __forceinline__ T sell_split_entry(T (*part)[BR][kSellPad], int e) {
 template <int BR, int BC, typename T>
 struct KSpmvSellSplit {
   static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
@@ -612,6 +669,7 @@ struct KSpmvSellSplit {
 template <int BR, typename T>
 struct KSmoothSellSplit {
   static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
     int64_t nbr;
@@ -703,6 +761,7 @@ __device__ __forceinline__ void d_spmv_rows(int64_t nbr, const int32_t *__restri
 template <int BR, int B0, int B1, int B2, int H>
 struct KSpmvRows {
   static constexpr int kMaxThreads = (H == 1 ? 64 : 32 * H);
+  static constexpr bool kFp64 = true;
   struct Args {
     int64_t nbr;
     const int32_t *sp;
@@ -740,6 +799,7 @@ __device__ __forceinline__ void d_smooth(int64_t nbr, const int32_t *__restrict_
 template <int BR, typename T, int U>
 struct KSmoothSell {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr int kMinBlocks = BR <= 3 ? 8 : 1;  // multi-system form: <= 32 registers
   struct Args {
     int64_t nbr;
@@ -806,6 +866,7 @@ __device__ __forceinline__ void d_gs_color(int64_t r0, int64_t r1, const int32_t
 template <int BR, typename T, int G>
 struct KGsColor {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   struct Args {
     int64_t r0;
     int64_t r1;
@@ -873,6 +934,7 @@ __device__ __forceinline__ void d_gs_small(int nc, int64_t n, const int32_t *__r
 template <int BR, typename T, int G>
 struct KGsSmall {
   static constexpr int kMaxThreads = kGsCtaThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
   struct Args {
     int nc;
     int64_t n;
@@ -910,7 +972,7 @@ struct KInvApply {
     const int row = bid * (blockDim.x / 32) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const double *a = p.inv + (int64_t)row * p.n;
-    const double a0 = row < p.n && lane < p.n ? __ldg(a + lane) : 0.0;
+    const double a0 = row < p.n && lane < p.n ? ld_pin(a + lane) : 0.0;
     wait();
     for (int j = threadIdx.x; j < p.n; j += blockDim.x) bs[j] = (double)p.b[j];
     __syncthreads();
@@ -1415,6 +1477,7 @@ __device__ __forceinline__ void d_mdot(const double *__restrict__ V, int64_t ldv
 }
 struct KMdot {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = true;
   struct Args {
     const double *V;
     int64_t ldv;
@@ -1461,6 +1524,7 @@ __device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_
 }
 struct KCgsFused {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = true;
   struct Args {
     const double *V;
     int64_t ldv;
@@ -1486,6 +1550,7 @@ __device__ __forceinline__ void d_reduce_partials(const double *__restrict__ par
 }
 struct KReducePartials {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = true;
   struct Args {
     const double *partial;
     int k;
@@ -1519,6 +1584,7 @@ __device__ __forceinline__ void d_cgs_update(const double *__restrict__ V, int64
 }
 struct KCgsUpdate {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = true;
   struct Args {
     const double *V;
     int64_t ldv;
@@ -1550,6 +1616,7 @@ __device__ __forceinline__ void d_gemv_add(const double *__restrict__ Z, int64_t
 }
 struct KGemvAdd {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = true;
   struct Args {
     const double *Z;
     int64_t ldz;
@@ -1789,8 +1856,9 @@ double fp64_rate(cudaStream_t s) {
 
 void set_launch_hook(LaunchHook *h) { g_hook = h; }
 void set_recorder(Recorder *r) { g_rec = r; }
-void set_pdl(unsigned max_grid) {
+void set_pdl(unsigned max_grid, unsigned max_grid64) {
   g_pdl = max_grid;
+  g_pdl64 = max_grid64;
   g_pdl_prev = nullptr;
 }
 void pdl_break() { g_pdl_prev = nullptr; }

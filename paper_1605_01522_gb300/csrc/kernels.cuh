@@ -81,9 +81,10 @@ struct Recorder {
   std::vector<RecOp> ops;
 };
 void set_recorder(Recorder *r);
-// this thread's solve-phase launches of at most max_grid CTAs overlap the end
-// of their predecessor in the stream (programmatic dependent launch); 0: none
-void set_pdl(unsigned max_grid);
+// this thread's solve-phase launches of at most max_grid CTAs (max_grid64:
+// kernels bound by the FP64 pipe) overlap the end of their predecessor in the
+// stream (programmatic dependent launch); 0, 0: none
+void set_pdl(unsigned max_grid, unsigned max_grid64);
 // the caller queued something other than a kernel on a stream: the next
 // launch waits for it the ordinary way
 void pdl_break();

@@ -157,13 +157,41 @@ struct PinnedCache {
 // never destroyed (the CUDA runtime may be gone at process exit)
 static PinnedCache &g_pinned = *new PinnedCache();
 
-// Layout autotuning: matrices with at least kTuneMinRows block rows are built
-// in both layouts (SELL-32, one thread per block row, with 2, 4 or 8 block
-// slots in flight; plain BSR, one warp per block row), each timed with CUDA
-// events, and the fastest is kept.  Smaller
-// matrices are latency bound and take the warp layout.  Decisions are cached
-// per (block shape, rows, blocks, precision) for the life of the process.
-constexpr int64_t kTuneMinRows = 2048;
+// Layouts.  Matrices with at least kTuneMinRows block rows (kTuneMinRowsBatch
+// in setups tuned for batches) are built in both layouts (SELL-32 with 2, 4 or
+// 8 slots in flight or several threads per block row; plain BSR, 8 to 32 lanes
+// per block row), each timed with CUDA events, and the fastest is kept;
+// decisions are cached per (block shape, rows, blocks, precision) for the life
+// of the process.  Smaller ones follow a rule (small_layout): their few
+// microseconds are less than event timings resolve, so the choice, and a
+// solve by up to 15 %, changed from process to process, and building both
+// layouts made their setups longer.
+constexpr int64_t kTuneMinRows = 131072;
+constexpr int64_t kTuneMinRowsBatch = 2048;
+
+// Threads per block row of a SELL-32 matrix of nbr rows of avg blocks: 8 for
+// long rows, 4 for short ones, halved while the matrix would take more than
+// 9,000 of the 9,728 warps that the GPU holds (timed best: 8 at 13,824 rows, 4
+// at 39,304 to 68,921).
+static int sell_split(int64_t nbr, double avg) {
+  int h = avg > 16.0 ? 8 : 4;
+  while (h > 1 && (nbr + 31) / 32 * h > 9000) h /= 2;
+  return h;
+}
+
+// The rule: 0 plain BSR, else SELL-32 with that many threads per row.  Plain
+// BSR puts 8 to 32 lanes on a row and so spreads few rows best (whole solves,
+// SELL-32 / plain BSR: 1,089 rows 1.95 / 1.71 ms, 4,851 rows 29.4 / 27.6, 13,824
+// rows 14.4 / 13.5); from 16,384 rows on SELL-32 fills the SMs with fewer
+// instructions (50,653 rows FP64 24.0 / 30.0 ms, 68,921 rows 18.3 / 19.4), from
+// 8,192 for short rows (prolongators, 4 blocks), which leave half the lanes
+// of a group idle (13,824 rows 13.4 / 13.5).  Rows of over 128 blocks and
+// blocks above 3x6 stay plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
+static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb) {
+  const double avg = nbr ? (double)nnzb / (double)nbr : 0.0;
+  if (br * bc > 18 || avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : 16384)) return 0;
+  return sell_split(nbr, avg);
+}
 
 static dev::Sell upload_layout(Arena &ar, const HBsr &A, bool want64, bool want32, int kind) {
   dev::Sell S;
@@ -333,6 +361,8 @@ static dev::Sell upload_layout_dev(Arena &ar, const RawDev *const *src, int nsrc
   return S;
 }
 
+// time of one product: the best of three event pairs around enough launches
+// (up to 8) that the events (about 5 us) do not hide the differences
 template <typename T> static float time_spmv(const dev::Sell &S, cudaStream_t st) {
   T *x = nullptr, *y = nullptr;
   MFS_CUDA(cudaMallocAsync((void **)&x, (size_t)std::max<int64_t>(1, S.ncols()) * sizeof(T), st));
@@ -342,14 +372,16 @@ template <typename T> static float time_spmv(const dev::Sell &S, cudaStream_t st
   MFS_CUDA(cudaEventCreate(&e0));
   MFS_CUDA(cudaEventCreate(&e1));
   float best = 1e30f;
+  int m = 1;
   for (int rep = 0; rep < 4; ++rep) {
     MFS_CUDA(cudaEventRecord(e0, st));
-    dev::spmv<T>(S, x, y, T(1), T(0), nullptr, st);
+    for (int k = 0; k < m; ++k) dev::spmv<T>(S, x, y, T(1), T(0), nullptr, st);
     MFS_CUDA(cudaEventRecord(e1, st));
     MFS_CUDA(cudaEventSynchronize(e1));
     float ms = 0.f;
     MFS_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-    if (rep > 0) best = std::min(best, ms);
+    if (rep > 0) best = std::min(best, ms / (float)m);
+    else m = ms > 0.1f ? 1 : ms > 0.03f ? 3 : 8;  // the first product also warms up
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -367,8 +399,7 @@ static thread_local int g_layout_tune = 0;
 // Layout candidates of the autotuner: 0 SELL-32 with 2 slots in flight,
 // 1 with 4, 2 plain BSR with one warp per row, 3 SELL-32 with 8 slots in
 // flight (only for blocks of at most 3 entries, whose rows are short on bytes),
-// 4, 5, 6 SELL-32 with 2, 4, 8 threads per row (the two that bring the matrix
-// closest to, but not far above, the 9,728 warps that the GPU holds; tuning
+// 4, 5, 6 SELL-32 with 2, 4, 8 threads per row (the one of sell_split; tuning
 // for batches leaves them out, other systems fill the GPU there).
 constexpr int kTuneCands = 7;
 static int tune_pick(const dev::Sell &a, const dev::Sell &b, bool want32, cudaStream_t st) {
@@ -389,9 +420,8 @@ static int tune_pick(const dev::Sell &a, const dev::Sell &b, bool want32, cudaSt
   for (int c = 4; c < kTuneCands; ++c) {
     dev::Sell ah = a;
     ah.split = 1 << (c - 3);
-    const int64_t warps = a.nslices * ah.split;
     t[c] = 1e30f;
-    if (g_layout_tune == 1 || warps > 20000 || (warps < 5000 && ah.split < 4)) continue;
+    if (g_layout_tune == 1 || ah.split != sell_split(a.nbr, (double)a.nnzb / (double)a.nbr)) continue;
     t[c] = want32 ? time_spmv<float>(ah, st) : time_spmv<double>(ah, st);
   }
   int best = 0;
@@ -420,7 +450,12 @@ static dev::Sell tune_keep(Arena &ar, dev::Sell &a, dev::Sell &b, int best) {
 }
 
 static dev::Sell upload_sell(Arena &ar, const HBsr &A, bool want64, bool want32) {
-  if (A.nbr < kTuneMinRows) return upload_layout(ar, A, want64, want32, 1);
+  if (A.nbr < (g_layout_tune == 1 ? kTuneMinRowsBatch : kTuneMinRows)) {
+    const int h = small_layout(A.br, A.bc, A.nbr, A.nnzb());
+    dev::Sell S = upload_layout(ar, A, want64, want32, h ? 0 : 1);
+    if (h) S.split = h;
+    return S;
+  }
   const auto key = std::make_tuple(A.br, A.bc, (int64_t)A.nbr, (int64_t)A.nnzb(), (want32 ? 1 : 0) + 2 * g_layout_tune);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -457,7 +492,12 @@ static dev::Sell upload_sell(Arena &ar, const HBsr &A, bool want64, bool want32)
 // the candidate layouts built on the device.
 static dev::Sell upload_sell_dev(Arena &ar, const RawDev &A, bool want64, bool want32, cudaStream_t st) {
   const RawDev *src[1] = {&A};
-  if (A.nbr < kTuneMinRows) return upload_layout_dev(ar, src, 1, want64, want32, 1, st);
+  if (A.nbr < (g_layout_tune == 1 ? kTuneMinRowsBatch : kTuneMinRows)) {
+    const int h = small_layout(A.br, A.bc, A.nbr, A.nnzb);
+    dev::Sell S = upload_layout_dev(ar, src, 1, want64, want32, h ? 0 : 1, st);
+    if (h) S.split = h;
+    return S;
+  }
   const auto key = std::make_tuple(A.br, A.bc, (int64_t)A.nbr, (int64_t)A.nnzb, (want32 ? 1 : 0) + 2 * g_layout_tune);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -1336,18 +1376,24 @@ static std::atomic<int> g_solves_running{0};
 
 // One solve-phase call: counted in g_solves_running, and its launches made
 // programmatic dependent launches as mfs_params.pdl says.  The automatic
-// choice: every launch of a small system, the launches of at most 160 CTAs
-// (coarse levels, reductions) of a larger one - its big launches measured
-// slower that way - and only while the call runs alone (16 concurrent solves
-// of small systems measured 2 % slower with them).
+// choice: every launch, but of the kernels that the FP64 pipe bounds only
+// those of at most 160 CTAs (a CTA per SM: see K::kFp64 in kernels.cu; with all
+// of them the 64^3 box took 59.6 instead of 57.3 ms without any, with this
+// rule 55.8; the 23^3 box AMG(BGS) 14.6 without, 12.3 with it), and only while the
+// call runs alone (16 concurrent solves of small systems measured 2 % slower
+// with them).
 struct SolvePhase {
   explicit SolvePhase(const mfs_handle *h) {
     const bool alone = ++g_solves_running == 1;
     const int p = h->prm.pdl;
-    dev::set_pdl(p == 1 ? ~0u : p > 1 ? (unsigned)p : (p == -1 && alone) ? (h->n <= 65536 ? ~0u : 160u) : 0u);
+    unsigned g = 0, g64 = 0;
+    if (p == 1) g = g64 = ~0u;
+    else if (p > 1) g = g64 = (unsigned)p;
+    else if (p == -1 && alone) g = ~0u, g64 = 160u;
+    dev::set_pdl(g, g64);
   }
   ~SolvePhase() {
-    dev::set_pdl(0);
+    dev::set_pdl(0, 0);
     --g_solves_running;
   }
 };

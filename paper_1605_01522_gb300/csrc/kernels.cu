@@ -581,10 +581,10 @@ constexpr int kSellSplitMax = 8;
 constexpr int kSellPad = 33;  // row pitch of the partial sums (bank conflicts)
 
 template <int BR, int BC, typename T, class W>
-__device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__restrict__ sp,
-                                                const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
-                                                const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
-                                                W wait, T (*part)[BR][kSellPad]) {
+__device__ __forceinline__ void sell_split_row(int64_t nbr, const int32_t *__restrict__ sp,
+                                               const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
+                                               const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
+                                               W wait, T (&acc)[BR]) {
   const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, H = blockDim.x >> 5;
   const int64_t row = slice * 32 + lane;
   const int64_t base = ld_pin(sp + slice);
@@ -593,7 +593,7 @@ __device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__re
   const T *vp = val + base * (BR * BC * 32) + lane;
   // first slot: before the wait (see k_solo)
   int64_t c = 0;
-  T v0[BR * BC], acc[BR];
+  T v0[BR * BC];
 #pragma unroll
   for (int e = 0; e < BR * BC; ++e) v0[e] = T(0);
   if (h < len) {
@@ -625,8 +625,17 @@ __device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__re
 #pragma unroll
       for (int q = 0; q < BC; ++q) acc[r] += __ldg(v + (r * BC + q) * 32) * xv[q];
   }
+}
+
+template <int BR, int BC, typename T, class W>
+__device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__restrict__ sp,
+                                                const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
+                                                const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
+                                                W wait, T (*part)[BR][kSellPad]) {
+  T acc[BR];
+  sell_split_row<BR, BC, T>(nbr, sp, rl, col, val, x, slice, wait, acc);
 #pragma unroll
-  for (int r = 0; r < BR; ++r) part[h][r][lane] = acc[r];
+  for (int r = 0; r < BR; ++r) part[threadIdx.x >> 5][r][threadIdx.x & 31] = acc[r];
   __syncthreads();
 }
 
@@ -695,6 +704,142 @@ struct KSmoothSellSplit {
       const T dd = a.c1 * a.d[i] + a.c2 * a.dinv[i] * res;
       a.d[i] = dd;
       a.xout[i] = a.x[i] + dd;
+    }
+  }
+};
+
+// Sums of products with their V-cycle epilogue (spmv_terms).  The couplings,
+// residuals and first smoothing steps of a small or mid-size level are
+// launches of 2 to 4 us whose work takes a fraction of that; one launch does
+// what 2 to 4 did (and the vectors in between are written and read once less).
+template <typename T> struct TermArgs {
+  const int32_t *rp, *rl, *col;  // rp: slice offsets in SELL-32
+  const T *val, *x;
+  int bc;
+};
+template <typename T> struct EpiArgs {
+  T alpha, beta, c1, c2;
+  const T *z, *dinv, *x;  // x: kRowSmooth's vector of the level
+  T *y, *d, *xout;
+  int mode;
+};
+// operands of one entry, loaded ahead of its sum
+template <typename T> struct EpiVals {
+  T z, dinv, d, x;
+};
+template <bool SM, typename T>
+__device__ __forceinline__ EpiVals<T> epi_load(const EpiArgs<T> &e, int64_t i) {
+  EpiVals<T> v;
+  if constexpr (SM) {
+    v.z = e.z[i];
+    v.dinv = e.dinv[i];
+    v.d = e.d[i];
+    v.x = e.x[i];
+  } else {
+    v.z = e.mode == kRowSub ? e.y[i] : e.z != nullptr ? e.z[i] : T(0);
+    v.dinv = e.mode != kRowPlain ? e.dinv[i] : T(0);
+  }
+  return v;
+}
+// s: the sum (SM: without the last term), t: the last term (SM)
+template <bool SM, typename T>
+__device__ __forceinline__ void epi_store(const EpiArgs<T> &e, int64_t i, const EpiVals<T> &v, T s, T t) {
+  if constexpr (SM) {
+    const T c = v.z - s;
+    const T res = c - t;
+    const T dd = e.c1 * v.d + e.c2 * v.dinv * res;
+    e.y[i] = c;
+    e.d[i] = dd;
+    e.xout[i] = v.x + dd;
+  } else if (e.mode == kRowSub) {
+    e.y[i] = v.z - v.dinv * s;
+  } else {
+    const T y = e.z != nullptr ? e.alpha * s + e.beta * v.z : e.alpha * s;
+    e.y[i] = y;
+    if (e.mode == kRowFirst) {
+      const T dd = e.c2 * v.dinv * y;
+      e.d[i] = dd;
+      e.xout[i] = dd;
+    }
+  }
+}
+
+#define MFS_BC_SWITCH(BCV, CALL)                     \
+  switch (BCV) {                                     \
+    case 1: { constexpr int BC_ = 1; CALL; } break;  \
+    case 2: { constexpr int BC_ = 2; CALL; } break;  \
+    case 3: { constexpr int BC_ = 3; CALL; } break;  \
+    default: { constexpr int BC_ = 6; CALL; } break; \
+  }
+
+template <int BR, typename T, bool SM>
+struct KTermsBsr {
+  static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
+  static constexpr bool kEarly = true;
+  struct Args {
+    int64_t nbr;
+    int nt, ls;
+    TermArgs<T> t[kMaxTerms];
+    EpiArgs<T> e;
+  };
+  template <class W> static __device__ __forceinline__ void run(const Args &a, int bid, int nb, W wait) {
+    const int64_t row = ((int64_t)bid * blockDim.x + threadIdx.x) >> a.ls;
+    const int gl = threadIdx.x & ((1 << a.ls) - 1);
+    const bool act = row < a.nbr, own = act && sum_owner<BR>(gl, a.ls);
+    const int64_t i = row * BR + sum_entry<BR>(gl, a.ls);
+    T acc[BR], last[BR];
+    MFS_BC_SWITCH(a.t[0].bc, (bsr_row<BR, BC_, T>(a.t[0].rp, a.t[0].col, a.t[0].val, a.t[0].x, row, act, gl, a.ls,
+                                                  wait, acc)));
+    for (int k = 1; k < a.nt; ++k) {
+      MFS_BC_SWITCH(a.t[k].bc, (bsr_row<BR, BC_, T>(a.t[k].rp, a.t[k].col, a.t[k].val, a.t[k].x, row, act, gl, a.ls,
+                                                    NoWait(), last)));
+      if (!SM || k + 1 < a.nt)
+#pragma unroll
+        for (int r = 0; r < BR; ++r) acc[r] += last[r];
+    }
+    EpiVals<T> v{};
+    if (own) v = epi_load<SM, T>(a.e, i);
+    const T s = group_sum<BR, T>(acc, gl, a.ls);
+    T t = T(0);
+    if constexpr (SM) t = group_sum<BR, T>(last, gl, a.ls);
+    if (own) epi_store<SM, T>(a.e, i, v, s, t);
+  }
+};
+
+template <int BR, typename T, bool SM>
+struct KTermsSell {
+  static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr bool kFp64 = sizeof(T) == 8;
+  static constexpr bool kEarly = true;
+  using Args = typename KTermsBsr<BR, T, SM>::Args;  // ls unused
+  template <class W> static __device__ __forceinline__ void run(const Args &a, int bid, int nb, W wait) {
+    __shared__ T part[kSellSplitMax][BR][kSellPad];
+    __shared__ T part2[SM ? kSellSplitMax : 1][BR][kSellPad];
+    const int lane = threadIdx.x & 31, h = threadIdx.x >> 5;
+    T acc[BR], last[BR];
+    MFS_BC_SWITCH(a.t[0].bc, (sell_split_row<BR, BC_, T>(a.nbr, a.t[0].rp, a.t[0].rl, a.t[0].col, a.t[0].val,
+                                                         a.t[0].x, bid, wait, acc)));
+    for (int k = 1; k < a.nt; ++k) {
+      MFS_BC_SWITCH(a.t[k].bc, (sell_split_row<BR, BC_, T>(a.nbr, a.t[k].rp, a.t[k].rl, a.t[k].col, a.t[k].val,
+                                                           a.t[k].x, bid, NoWait(), last)));
+      if (!SM || k + 1 < a.nt)
+#pragma unroll
+        for (int r = 0; r < BR; ++r) acc[r] += last[r];
+    }
+#pragma unroll
+    for (int r = 0; r < BR; ++r) {
+      part[h][r][lane] = acc[r];
+      if constexpr (SM) part2[h][r][lane] = last[r];
+    }
+    __syncthreads();
+    const int64_t i0 = (int64_t)bid * 32 * BR, n = a.nbr * BR;
+    for (int e = threadIdx.x; e < 32 * BR && i0 + e < n; e += blockDim.x) {
+      const EpiVals<T> v = epi_load<SM, T>(a.e, i0 + e);
+      const T s = sell_split_entry<BR, T>(part, e);
+      T t = T(0);
+      if constexpr (SM) t = sell_split_entry<BR, T>(part2, e);
+      epi_store<SM, T>(a.e, i0 + e, v, s, t);
     }
   }
 };
@@ -2032,6 +2177,65 @@ void smooth_first(int64_t n, const T *dinv, const T *b, T *x, T *d, T c2, cudaSt
   HookScope hs(s, K_VECTOR, 4.0 * n * sizeof(T), 1, n, 2.0 * n);
   go<KSmoothFirst<T>>(ew_grid(n), kThreads, 0, s, {n, dinv, b, x, d, c2});
 }
+
+template <typename T> bool rows_fusable(const RowTerm<T> *t, int n) {
+  if (n < 1 || n > kMaxTerms) return false;
+  for (int k = 0; k < n; ++k) {
+    const Sell &A = *t[k].A;
+    if (A.nbr == 0 || A.nbr != t[0].A->nbr || A.br != t[0].A->br || A.kind != t[0].A->kind) return false;
+    if (A.br != 1 && A.br != 2 && A.br != 3 && A.br != 6) return false;
+    if (A.bc != 1 && A.bc != 2 && A.bc != 3 && A.bc != 6) return false;
+    // one thread per row (large systems: the launches are long) and one CTA per row stay separate
+    if (A.kind == 0 ? A.split <= 1 : cta_rows<T>(A)) return false;
+  }
+  return true;
+}
+template bool rows_fusable<float>(const RowTerm<float> *, int);
+template bool rows_fusable<double>(const RowTerm<double> *, int);
+
+template <int BR, typename T, bool SM>
+static void terms_launch(const RowTerm<T> *t, int n, const RowOut<T> &o, int split, int ls, cudaStream_t s) {
+  typename KTermsBsr<BR, T, SM>::Args a{};
+  const Sell &A = *t[0].A;
+  a.nbr = A.nbr;
+  a.nt = n;
+  a.ls = ls;
+  for (int k = 0; k < n; ++k) {
+    const Sell &M = *t[k].A;
+    a.t[k] = {M.sp, M.rl, M.col, vals<T>(M), t[k].x, M.bc};
+  }
+  a.e = {o.alpha, o.beta, o.c1, o.c2, o.z, o.dinv, SM ? t[n - 1].x : nullptr, o.y, o.d, o.xout, o.mode};
+  if (A.kind == 0) {
+    go<KTermsSell<BR, T, SM>>((unsigned)A.nslices, 32 * split, 0, s, a);
+  } else {
+    const unsigned th = bsr_threads(A.nbr << ls);
+    go<KTermsBsr<BR, T, SM>>(grid_for(A.nbr << ls, th), th, 0, s, a);
+  }
+}
+
+template <typename T> void spmv_terms(const RowTerm<T> *t, int n, const RowOut<T> &o, cudaStream_t s) {
+  const Sell &A = *t[0].A;
+  double bytes = 0.0, flops = 0.0;
+  int split = 1, ls = 0;
+  for (int k = 0; k < n; ++k) {
+    const Sell &M = *t[k].A;
+    bytes += matrix_bytes<T>(M) + (double)sizeof(T) * M.ncols();
+    flops += 2.0 * M.nnzb * M.br * M.bc;
+    split = std::max(split, M.split);
+    ls = std::max(ls, M.kind == 1 ? bsr_ls<T>(M) : 0);
+  }
+  const double vecs = o.mode == kRowSmooth ? 6.0 : o.mode == kRowFirst ? 4.0 + (o.z ? 1 : 0) : o.mode == kRowSub ? 3.0 : o.z ? 2.0 : 1.0;
+  HookScope hs(s, o.mode == kRowSmooth ? K_SMOOTH : K_SPMV, bytes + sizeof(T) * vecs * A.nrows(),
+               (A.kind == 0 ? 11000 : 10000) + A.br * 100 + n * 10 + (sizeof(T) == 8 ? 1 : 0), A.nbr,
+               flops + vecs * A.nrows());
+  if (o.mode == kRowSmooth) {
+    MFS_SQUARE_DISPATCH(A.br, (terms_launch<BR_, T, true>(t, n, o, split, ls, s)));
+  } else {
+    MFS_SQUARE_DISPATCH(A.br, (terms_launch<BR_, T, false>(t, n, o, split, ls, s)));
+  }
+}
+template void spmv_terms<float>(const RowTerm<float> *, int, const RowOut<float> &, cudaStream_t);
+template void spmv_terms<double>(const RowTerm<double> *, int, const RowOut<double> &, cudaStream_t);
 
 #define MFS_GS_G_DISPATCH(GV, CALL)                              \
   switch (GV) {                                                  \

@@ -44,7 +44,8 @@ enum KernelClass { K_SPMV = 0, K_SMOOTH = 1, K_VECTOR = 2, K_COARSE = 3, K_ARNOL
 // layout*1000 + br*100 + bc*10 + (float64 ? 1 : 0) with layout 0 SELL-32,
 // 1 warp BSR, 2 merged rows, 3 SELL-32 with 4 slots in flight, 4 / 5 / 6 the
 // Gauss-Seidel colour kernels on SELL-32 / warp BSR / SELL-32 x4, 7 one CTA per
-// BSR row, 8 SELL-32 with several threads per row; otherwise a small id.
+// BSR row, 8 SELL-32 with several threads per row, 10 / 11 a sum of bc products in one
+// launch (plain BSR / SELL-32); otherwise a small id.
 // rows = block rows (sparse kernels) or vector length.
 struct LaunchHook {
   // returns false when this launch is not to be recorded (after() is then skipped)
@@ -110,6 +111,34 @@ struct DenseLU {
 // y = alpha * A x + beta * z   (z may alias y or be null when beta == 0)
 template <typename T>
 void spmv(const Sell &A, const T *x, T *y, T alpha, T beta, const T *z, cudaStream_t s);
+
+// One launch for a sum of products over one row space, s = sum_t A_t x_t
+// (n <= kMaxTerms matrices with the same block rows), and what the V-cycles
+// do with it, per entry:
+//   kRowPlain   y = alpha s + beta z                      (z may be null)
+//   kRowFirst   the same, then d = xout = c2 dinv y       (first smoothing step from zero)
+//   kRowSmooth  s without the last term: y = z - s; with it (the level's own
+//               matrix, x its vector): r = y - A x; d = c1 d + c2 dinv r; xout = x + d
+//   kRowSub     y -= dinv s
+// rows_fusable: the matrices' layouts allow it (else the caller runs the steps
+// one by one).
+constexpr int kMaxTerms = 4;
+enum RowMode { kRowPlain = 0, kRowFirst = 1, kRowSmooth = 2, kRowSub = 3 };
+template <typename T> struct RowTerm {
+  const Sell *A = nullptr;
+  const T *x = nullptr;
+};
+template <typename T> struct RowOut {
+  int mode = kRowPlain;
+  T alpha = T(1), beta = T(0);
+  const T *z = nullptr;
+  T *y = nullptr;
+  const T *dinv = nullptr;
+  T *d = nullptr, *xout = nullptr;
+  T c1 = T(0), c2 = T(0);
+};
+template <typename T> bool rows_fusable(const RowTerm<T> *t, int n);
+template <typename T> void spmv_terms(const RowTerm<T> *t, int n, const RowOut<T> &o, cudaStream_t s);
 
 // All blocks of one block row of fields that share one sparsity pattern,
 // merged: each slot holds [A_i0 | A_i1 | A_i2] (br x (b0+b1+b2), row-major,

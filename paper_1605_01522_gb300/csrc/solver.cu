@@ -185,11 +185,13 @@ static int sell_split(int64_t nbr, double avg) {
 // rows 14.4 / 13.5); from 16,384 rows on SELL-32 fills the SMs with fewer
 // instructions (50,653 rows FP64 24.0 / 30.0 ms, 68,921 rows 18.3 / 19.4), from
 // 8,192 for short rows (prolongators, 4 blocks), which leave half the lanes
-// of a group idle (13,824 rows 13.4 / 13.5).  Rows of over 128 blocks and
-// blocks above 3x6 stay plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
+// of a group idle (13,824 rows 13.4 / 13.5), from 49,152 for rows of over 32
+// blocks, which a lane walks longest (20,261 rows of 105 1x1 blocks 15.9 / 10.4
+// us a product, 68,921 of 114 16.2 / 20.3).  Rows of over 128 blocks and blocks
+// above 3x6 stay plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
 static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb) {
   const double avg = nbr ? (double)nnzb / (double)nbr : 0.0;
-  if (br * bc > 18 || avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : 16384)) return 0;
+  if (br * bc > 18 || avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : avg <= 32.0 ? 16384 : 49152)) return 0;
   return sell_split(nbr, avg);
 }
 
@@ -741,6 +743,12 @@ template <typename T> struct Precond {
   int kind = 0, nf = 0, order = 0, sweeps = 1;
   int smoother = MFS_CHEBYSHEV, gs_sweeps = 1;
   bool use_tail = false;  // one-CTA V-cycle tails where they apply (mfs_params.vcycle_tail)
+  // sums of products and their epilogues in one launch (dev::spmv_terms).  Not
+  // for handles tuned for batches: there the merged launches fill the GPU and
+  // the wider kernels' registers cost more than the launches (96 small systems
+  // 14.8 instead of 14.3 ms).
+  bool fuse = true;
+  bool fusable(const dev::RowTerm<T> *t, size_t n) const { return fuse && dev::rows_fusable<T>(t, (int)n); }
   T gs_omega = T(0.79);
   std::vector<int64_t> fsize, foff;
   DGroup<T> g0, g1;
@@ -769,9 +777,14 @@ template <typename T> struct Precond {
     }
   }
 
+  // Where the first step from zero writes x, so that the last step ends in x
+  T *first_target(FL<T> &f, T *x) const { return ((int)f.c1.size() - 1) % 2 == 0 ? x : f.t; }
+
   // single-field smoother S^l_i; zero: x enters as 0; post: the application
-  // after the coarse correction (Gauss-Seidel then sweeps backward)
-  void smooth(FL<T> &f, const T *rhs, T *x, bool zero, bool post = false) {
+  // after the coarse correction (Gauss-Seidel then sweeps backward); done: the
+  // first step has been made already (into first_target(f, x), or f.t when x
+  // was not zero)
+  void smooth(FL<T> &f, const T *rhs, T *x, bool zero, bool post = false, bool done = false) {
     if (smoother == MFS_GS) {
       if (zero) dev::fill<T>(x, f.n, T(0), s);
       dev::gs_sweeps<T>(f.gs, f.dblk, rhs, x, gs_omega, gs_sweeps, post, s);
@@ -781,10 +794,13 @@ template <typename T> struct Precond {
     T *cur = x, *oth = f.t;
     int k0 = 0;
     if (zero) {
-      T *tgt = ((ns - 1) % 2 == 0) ? x : f.t;
-      dev::smooth_first<T>(f.n, f.dinv, rhs, tgt, f.d, f.c2[0], s);
+      T *tgt = first_target(f, x);
+      if (!done) dev::smooth_first<T>(f.n, f.dinv, rhs, tgt, f.d, f.c2[0], s);
       cur = tgt;
       oth = tgt == x ? f.t : x;
+      k0 = 1;
+    } else if (done) {
+      std::swap(cur, oth);
       k0 = 1;
     }
     for (int k = k0; k < ns; ++k) {
@@ -792,6 +808,69 @@ template <typename T> struct Precond {
       std::swap(cur, oth);
     }
     if (cur != x) dev::convert<T, T>(cur, x, f.n, s);
+  }
+
+  // y = rhs - sum_t A_t x_t (no terms: y is not written, rhs is returned); with
+  // `first` also the first smoothing step of that field from zero into x.
+  // One launch where the layouts allow it; *done says whether the first step
+  // was made.
+  const T *subtract(std::vector<dev::RowTerm<T>> &terms, const T *rhs, T *y, FL<T> *first = nullptr, T *x = nullptr,
+                    bool *done = nullptr) {
+    if (terms.empty()) return rhs;
+    if (fusable(terms.data(), terms.size())) {
+      dev::RowOut<T> o;
+      o.alpha = T(-1);
+      o.beta = T(1);
+      o.z = rhs;
+      o.y = y;
+      if (first) set_first(o, *first, x, done);
+      dev::spmv_terms<T>(terms.data(), (int)terms.size(), o, s);
+      return y;
+    }
+    for (auto &t : terms) {
+      dev::spmv<T>(*t.A, t.x, y, T(-1), T(1), rhs, s);
+      rhs = y;
+    }
+    return y;
+  }
+  void set_first(dev::RowOut<T> &o, FL<T> &f, T *x, bool *done) {
+    if (smoother == MFS_GS || f.c1.empty()) return;
+    o.mode = dev::kRowFirst;
+    o.dinv = f.dinv;
+    o.d = f.d;
+    o.xout = first_target(f, x);
+    o.c2 = f.c2[0];
+    *done = true;
+  }
+  // restriction c.bv = R r of field i to level l + 1, with the first smoothing
+  // step of that level where it has one
+  bool restrict_to(DGroup<T> &g, int i, int l, const T *r, bool smoothed) {
+    FL<T> &f = g.lv[l][i], &c = g.lv[l + 1][i];
+    dev::RowTerm<T> t{&f.R, r};
+    bool done = false;
+    if (smoothed && smoother != MFS_GS && fusable(&t, 1)) {
+      dev::RowOut<T> o;
+      o.y = c.bv;
+      set_first(o, c, c.xv, &done);
+      dev::spmv_terms<T>(&t, 1, o, s);
+    } else {
+      dev::spmv<T>(f.R, r, c.bv, T(1), T(0), nullptr, s);
+    }
+    return done;
+  }
+  // x -= dinv A v  (t: scratch)
+  void sub_diag(const dev::Sell &A, const T *v, const T *dinv, T *x, T *t, int64_t n) {
+    dev::RowTerm<T> term{&A, v};
+    if (fusable(&term, 1)) {
+      dev::RowOut<T> o;
+      o.mode = dev::kRowSub;
+      o.dinv = dinv;
+      o.y = x;
+      dev::spmv_terms<T>(&term, 1, o, s);
+      return;
+    }
+    dev::spmv<T>(A, v, t, T(1), T(0), nullptr, s);
+    dev::axpy_diag<T>(x, dinv, t, n, s);
   }
 
   // the level above the coarsest, small enough that one CTA runs the rest of
@@ -808,8 +887,12 @@ template <typename T> struct Precond {
     return dev::tail_smem_bytes(A.nrows(), lu.n, sizeof(T)) <= 48 * 1024;
   }
 
-  // Algorithm 1 for field i of group g from level l, zero initial guess
-  void vcycle(DGroup<T> &g, int i, int l, const T *rhs, T *x) {
+  // level l of field i is smoothed by the step-by-step V-cycle
+  bool stepwise(const DGroup<T> &g, int i, int l) const { return l < g.L - 1 && !tail_ok(g, i, l); }
+
+  // Algorithm 1 for field i of group g from level l, zero initial guess; done:
+  // the level's first smoothing step has been made
+  void vcycle(DGroup<T> &g, int i, int l, const T *rhs, T *x, bool done = false) {
     FL<T> &f = g.lv[l][i];
     if (l == g.L - 1) {
       dev::lu_solve<T>(g.cf[i], rhs, x, s);
@@ -820,10 +903,10 @@ template <typename T> struct Precond {
       return;
     }
     FL<T> &c = g.lv[l + 1][i];
-    smooth(f, rhs, x, true);
+    smooth(f, rhs, x, true, false, done);
     dev::spmv<T>(f.A, x, f.r, T(-1), T(1), rhs, s);
-    dev::spmv<T>(f.R, f.r, c.bv, T(1), T(0), nullptr, s);
-    vcycle(g, i, l + 1, c.bv, c.xv);
+    const bool next = restrict_to(g, i, l, f.r, stepwise(g, i, l + 1));
+    vcycle(g, i, l + 1, c.bv, c.xv, next);
     dev::spmv<T>(f.P, c.xv, x, T(1), T(1), x, s);
     smooth(f, rhs, x, false, true);
   }
@@ -841,9 +924,21 @@ template <typename T> struct Precond {
 
   // block solve of BGS: one V-cycle, or for the single-level BGS(GS) the
   // Gauss-Seidel sweeps from zero on the fine block
-  void leaf(DGroup<T> &g, int i, const T *rhs, T *x) {
+  void leaf(DGroup<T> &g, int i, const T *rhs, T *x, bool done) {
     if (kind == MFS_BGS_GS) smooth(g.lv[0][i], rhs, x, true, false);
-    else vcycle(g, i, 0, rhs, x);
+    else vcycle(g, i, 0, rhs, x, done);
+  }
+
+  // the coupling terms A_ij x_j of field i with the fields marked in nz
+  std::vector<dev::RowTerm<T>> couplings(const DGroup<T> &g, int l, int i, const std::vector<T *> &x,
+                                         const std::vector<char> &nz, bool self) {
+    std::vector<dev::RowTerm<T>> t;
+    for (int j = 0; j < g.nf; ++j) {
+      if (!nz[j] || (j == i && !self)) continue;
+      const dev::Sell *M = g.block(l, i, j);
+      if (M && M->nbr) t.push_back({M, x[j]});
+    }
+    return t;
   }
 
   // block Gauss-Seidel on level 0 of group g with V-cycle block solves
@@ -853,45 +948,59 @@ template <typename T> struct Precond {
       for (auto &seq : orders(order, g.nf))
         for (int i : seq) {
           FL<T> &f = g.lv[0][i];
-          const T *rhs = b[i];
-          for (int j = 0; j < g.nf; ++j) {
-            if (!nz[j]) continue;
-            const dev::Sell *M = g.block(0, i, j);
-            if (!M) continue;
-            dev::spmv<T>(*M, x[j], f.c, T(-1), T(1), rhs, s);
-            rhs = f.c;
-          }
-          if (!nz[i]) {
-            leaf(g, i, rhs, x[i]);
-            nz[i] = 1;
-          } else {
-            leaf(g, i, rhs, f.e);
-            dev::axpy<T>(x[i], f.e, T(1), f.n, s);
-          }
+          T *dst = nz[i] ? f.e : x[i];
+          bool done = false;
+          auto t = couplings(g, 0, i, x, nz, true);
+          const bool first = kind != MFS_BGS_GS && stepwise(g, i, 0);
+          const T *rhs = subtract(t, b[i], f.c, first ? &f : nullptr, dst, &done);
+          leaf(g, i, rhs, dst, done);
+          if (nz[i]) dev::axpy<T>(x[i], f.e, T(1), f.n, s);
+          nz[i] = 1;
         }
   }
 
   void mono_smooth(DGroup<T> &g, int l, const std::vector<const T *> &b, const std::vector<T *> &x, bool zero,
-                   bool post) {
+                   bool post, const std::vector<char> &firsts) {
     std::vector<char> nz(g.nf, zero ? 0 : 1);
     for (int sw = 0; sw < sweeps; ++sw)
       for (auto &seq : orders(order, g.nf))
         for (int i : seq) {
           FL<T> &f = g.lv[l][i];
+          auto t = couplings(g, l, i, x, nz, false);
           const T *rhs = b[i];
-          for (int j = 0; j < g.nf; ++j) {
-            if (j == i || !nz[j]) continue;
-            const dev::Sell *M = g.block(l, i, j);
-            if (!M) continue;
-            dev::spmv<T>(*M, x[j], f.c, T(-1), T(1), rhs, s);
-            rhs = f.c;
+          // no couplings yet: the first step may have come with the restriction
+          bool done = !nz[i] && t.empty() && !firsts.empty() && firsts[i];
+          if (nz[i] && !t.empty() && smoother != MFS_GS && !f.c1.empty()) {
+            // couplings and the first step in one launch (b - sum A_ij x_j
+            // kept in f.c for the other steps)
+            t.push_back({&f.A, x[i]});
+            if (fusable(t.data(), t.size())) {
+              dev::RowOut<T> o;
+              o.mode = dev::kRowSmooth;
+              o.z = b[i];
+              o.y = f.c;
+              o.dinv = f.dinv;
+              o.d = f.d;
+              o.xout = f.t;
+              o.c1 = f.c1[0];
+              o.c2 = f.c2[0];
+              dev::spmv_terms<T>(t.data(), (int)t.size(), o, s);
+              rhs = f.c;
+              done = true;
+              t.clear();
+            } else {
+              t.pop_back();
+            }
           }
-          smooth(f, rhs, x[i], !nz[i], post);
+          if (!t.empty()) rhs = subtract(t, b[i], f.c, nz[i] ? nullptr : &f, x[i], &done);
+          smooth(f, rhs, x[i], !nz[i], post, done);
           nz[i] = 1;
         }
   }
 
-  void mono_cycle(DGroup<T> &g, int l, const std::vector<const T *> &b, const std::vector<T *> &x) {
+  // firsts: fields whose first smoothing step came with the restriction
+  void mono_cycle(DGroup<T> &g, int l, const std::vector<const T *> &b, const std::vector<T *> &x,
+                  const std::vector<char> &firsts = {}) {
     if (l == g.L - 1) {
       for (int i = 0; i < g.nf; ++i)
         if (b[i] != g.lv[l][i].bv)
@@ -902,30 +1011,31 @@ template <typename T> struct Precond {
           dev::convert<T, T>(g.lv[l][i].xv, x[i], g.lv[l][i].n, s);
       return;
     }
-    level_smooth(g, l, b, x, true);
+    level_smooth(g, l, b, x, true, firsts);
     std::vector<const T *> bc(g.nf);
     std::vector<T *> xc(g.nf);
+    std::vector<char> next(g.nf, 0);
+    const std::vector<char> all(g.nf, 1);
+    // the field that level l + 1 smooths first has no couplings there
+    const int lead = kind == MFS_AMG_SIMPLE ? -1 : orders(order, g.nf)[0][0];
     for (int i = 0; i < g.nf; ++i) {
       FL<T> &f = g.lv[l][i];
-      dev::spmv<T>(f.A, x[i], f.r, T(-1), T(1), b[i], s);
-      for (int j = 0; j < g.nf; ++j) {
-        if (j == i) continue;
-        const dev::Sell *M = g.block(l, i, j);
-        if (M) dev::spmv<T>(*M, x[j], f.r, T(-1), T(1), f.r, s);
-      }
-      dev::spmv<T>(f.R, f.r, g.lv[l + 1][i].bv, T(1), T(0), nullptr, s);
+      auto t = couplings(g, l, i, x, all, true);
+      subtract(t, b[i], f.r);
+      next[i] = restrict_to(g, i, l, f.r, i == lead && l + 1 < g.L - 1);
       bc[i] = g.lv[l + 1][i].bv;
       xc[i] = g.lv[l + 1][i].xv;
     }
-    mono_cycle(g, l + 1, bc, xc);
+    mono_cycle(g, l + 1, bc, xc, next);
     for (int i = 0; i < g.nf; ++i) dev::spmv<T>(g.lv[l][i].P, xc[i], x[i], T(1), T(1), x[i], s);
-    level_smooth(g, l, b, x, false);
+    level_smooth(g, l, b, x, false, {});
   }
 
   // pre-smoothing enters with x = 0, post-smoothing after the coarse correction
-  void level_smooth(DGroup<T> &g, int l, const std::vector<const T *> &b, const std::vector<T *> &x, bool zero) {
+  void level_smooth(DGroup<T> &g, int l, const std::vector<const T *> &b, const std::vector<T *> &x, bool zero,
+                    const std::vector<char> &firsts) {
     if (kind == MFS_AMG_SIMPLE) simple_smooth(g, l, b, x, zero, !zero);
-    else mono_smooth(g, l, b, x, zero, !zero);
+    else mono_smooth(g, l, b, x, zero, !zero, firsts);
   }
 
   // AMG(SIMPLE) level smoother: r = b - A x; one BGS sweep of the field
@@ -943,13 +1053,8 @@ template <typename T> struct Precond {
           continue;
         }
         FL<T> &f = g.lv[l][i];
-        dev::spmv<T>(f.A, x[i], f.r, T(-1), T(1), b[i], s);
-        for (int j = 0; j < g.nf; ++j) {
-          if (j == i) continue;
-          const dev::Sell *M = g.block(l, i, j);
-          if (M) dev::spmv<T>(*M, x[j], f.r, T(-1), T(1), f.r, s);
-        }
-        r[i] = f.r;
+        auto t = couplings(g, l, i, x, std::vector<char>(g.nf, 1), true);
+        r[i] = subtract(t, b[i], f.r);
       }
       std::vector<char> done(g.nf, 0);
       const int n1 = (int)G1.size();
@@ -957,36 +1062,32 @@ template <typename T> struct Precond {
         for (int jj : seq) {
           const int i = G1[jj];
           FL<T> &f = g.lv[l][i];
-          const T *rhs = r[i];
+          std::vector<dev::RowTerm<T>> t;
           for (int q : G1) {
             if (q == i || !done[q]) continue;
             const dev::Sell *M = g.block(l, i, q);
-            if (!M) continue;
-            dev::spmv<T>(*M, g.lv[l][q].e, f.c, T(-1), T(1), rhs, s);
-            rhs = f.c;
+            if (M && M->nbr) t.push_back({M, g.lv[l][q].e});
           }
-          if (!done[i]) {
-            smooth(f, rhs, f.e, true, post);
-            done[i] = 1;
-          } else {  // second visit of a symmetric sweep: correction form
-            smooth(f, rhs, f.e, false, post);
-          }
+          bool fd = false;
+          const T *rhs = subtract(t, r[i], f.c, done[i] ? nullptr : &f, f.e, &fd);
+          // second visit of a symmetric sweep: correction form
+          smooth(f, rhs, f.e, !done[i], post, fd);
+          done[i] = 1;
         }
-      const T *rhs2 = r[k];
+      std::vector<dev::RowTerm<T>> t2;
       for (int j : G1) {
         const dev::Sell *M = g.block(l, k, j);
-        if (!M) continue;
-        dev::spmv<T>(*M, g.lv[l][j].e, sk.c, T(-1), T(1), rhs2, s);
-        rhs2 = sk.c;
+        if (M && M->nbr) t2.push_back({M, g.lv[l][j].e});
       }
-      smooth(sk, rhs2, sk.e, true, post);
+      bool fd2 = false;
+      const T *rhs2 = subtract(t2, r[k], sk.c, &sk, sk.e, &fd2);
+      smooth(sk, rhs2, sk.e, true, post, fd2);
       for (int jj = 0; jj < n1; ++jj) {
         const int j = G1[jj];
         const dev::Sell *M = g.block(l, j, k);
         if (!M) continue;
         FL<T> &f = g.lv[l][j];
-        dev::spmv<T>(*M, sk.e, f.c, T(1), T(0), nullptr, s);
-        dev::axpy_diag<T>(f.e, ms_dtinv[l][jj], f.c, f.n, s);
+        sub_diag(*M, sk.e, ms_dtinv[l][jj], f.e, f.c, f.n);
       }
       for (int j : G1) {
         FL<T> &f = g.lv[l][j];
@@ -1022,29 +1123,34 @@ template <typename T> struct Precond {
       if (g0.mono) mono_cycle(g0, 0, b1, x1);
       else if (G1.size() == 1) vcycle(g0, 0, 0, b1[0], x1[0]);
       else bgs(g0, b1, x1);
-      // Schur right-hand side b_2 - A_21 dx_1
+      // Schur right-hand side b_2 - A_21 dx_1 (one Schur field: with the first
+      // smoothing step of its V-cycle)
+      bool done = false;
       for (size_t kk = 0; kk < G2.size(); ++kk) {
-        const T *rhs = b[G2[kk]];
+        std::vector<dev::RowTerm<T>> t;
         for (size_t jj = 0; jj < G1.size(); ++jj) {
           auto it = cross.find({G2[kk], G1[jj]});
-          if (it == cross.end()) continue;
-          dev::spmv<T>(it->second, x1[jj], sr2[kk], T(-1), T(1), rhs, s);
-          rhs = sr2[kk];
+          if (it != cross.end() && it->second.nbr) t.push_back({&it->second, x1[jj]});
         }
-        b2.push_back(rhs);
+        const bool first = G2.size() == 1 && stepwise(g1, 0, 0);
+        b2.push_back(subtract(t, b[G2[kk]], sr2[kk], first ? &g1.lv[0][0] : nullptr, x2[kk], &done));
       }
-      if (G2.size() == 1) vcycle(g1, 0, 0, b2[0], x2[0]);
+      if (G2.size() == 1) vcycle(g1, 0, 0, b2[0], x2[0], done);
       else bgs(g1, b2, x2);
       // update x_1 = dx_1 - A~11^-1 A_12 dx_2
       for (size_t jj = 0; jj < G1.size(); ++jj) {
-        bool any = false;
+        std::vector<std::pair<const dev::Sell *, const T *>> t;
         for (size_t kk = 0; kk < G2.size(); ++kk) {
           auto it = cross.find({G1[jj], G2[kk]});
-          if (it == cross.end()) continue;
-          dev::spmv<T>(it->second, x2[kk], st[jj], T(1), any ? T(1) : T(0), any ? st[jj] : nullptr, s);
-          any = true;
+          if (it != cross.end()) t.push_back({&it->second, x2[kk]});
         }
-        if (any) dev::axpy_diag<T>(x1[jj], dtinv[jj], st[jj], fsize[G1[jj]], s);
+        if (t.size() == 1) {
+          sub_diag(*t[0].first, t[0].second, dtinv[jj], x1[jj], st[jj], fsize[G1[jj]]);
+        } else if (!t.empty()) {
+          for (size_t q = 0; q < t.size(); ++q)
+            dev::spmv<T>(*t[q].first, t[q].second, st[jj], T(1), q ? T(1) : T(0), q ? st[jj] : nullptr, s);
+          dev::axpy_diag<T>(x1[jj], dtinv[jj], st[jj], fsize[G1[jj]], s);
+        }
       }
     }
   }
@@ -2412,6 +2518,7 @@ void upload_precond(mfs_handle *h, Arena &mat, Precond<T> &P, const std::map<std
   auto fine_sell = [&](int i, int j) { return h->A64.at({i, j}); };
   P.smoother = p.smoother;
   P.use_tail = p.vcycle_tail != 0;
+  P.fuse = p.layout_tune == 0;
   P.gs_sweeps = p.gs_sweeps;
   P.gs_omega = (T)p.gs_omega;
   if (p.precond == MFS_BGS_AMG || p.precond == MFS_AMG_BGS || p.precond == MFS_AMG_SIMPLE ||

@@ -270,19 +270,24 @@ __global__ void k_div_into(const double *__restrict__ w, double *__restrict__ v,
   if (i < n) v[i] = w[i] / *s;
 }
 
-// y = dinv .* (A x), one thread per block row
+// y = dinv .* (A x), one thread per row (a row's products in their order,
+// loads of four blocks in flight); BC: compile-time block columns, 0: any
+template <int BC>
 __global__ void k_dinv_spmv(BV A, const double *__restrict__ x, const double *__restrict__ dinv, double *__restrict__ y) {
-  const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t I = t / A.br;
   if (I >= A.nbr) return;
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  const int bs = A.br * A.bc;
+  const int r = (int)(t - I * A.br), bc = BC ? BC : A.bc;
+  const double *v = A.v + (int64_t)r * bc;
+  const int64_t bs = (int64_t)A.br * bc;
+  double acc = 0.0;
+#pragma unroll 4
   for (int a = A.rp[I]; a < A.rp[I + 1]; ++a) {
-    const double *blk = A.v + (int64_t)a * bs;
-    const double *xv = x + (int64_t)A.ci[a] * A.bc;
-    for (int r = 0; r < A.br; ++r)
-      for (int c = 0; c < A.bc; ++c) acc[r] += blk[r * A.bc + c] * xv[c];
+    const double *xv = x + (int64_t)A.ci[a] * bc;
+#pragma unroll
+    for (int c = 0; c < bc; ++c) acc += v[a * bs + c] * xv[c];
   }
-  for (int r = 0; r < A.br; ++r) y[I * A.br + r] = dinv[I * A.br + r] * acc[r];
+  y[t] = dinv[t] * acc;
 }
 
 __global__ void k_diag_inv(BV A, double *__restrict__ dinv, int *__restrict__ bad) {
@@ -316,7 +321,10 @@ double power_lambda_gpu(const DB &A, const double *dinv, uint64_t seed) {
   k_final_sqrt<<<1, 32, 0, gstream()>>>(part.p, 256, nrm.p);
   k_scale_by<<<nblocks(n), kT, 0, gstream()>>>(v.p, n, nrm.p);
   for (int it = 0; it < 10; ++it) {
-    k_dinv_spmv<<<nblocks(A.nbr), kT, 0, gstream()>>>(view(A), v.p, dinv, w.p);
+    if (A.bc == 1) k_dinv_spmv<1><<<nblocks(n), kT, 0, gstream()>>>(view(A), v.p, dinv, w.p);
+    else if (A.bc == 3) k_dinv_spmv<3><<<nblocks(n), kT, 0, gstream()>>>(view(A), v.p, dinv, w.p);
+    else if (A.bc == 6) k_dinv_spmv<6><<<nblocks(n), kT, 0, gstream()>>>(view(A), v.p, dinv, w.p);
+    else k_dinv_spmv<0><<<nblocks(n), kT, 0, gstream()>>>(view(A), v.p, dinv, w.p);
     k_sumsq_partial<<<256, kT, 0, gstream()>>>(w.p, n, part.p);
     k_final_sqrt<<<1, 32, 0, gstream()>>>(part.p, 256, nrm.p);
     k_div_into<<<nblocks(n), kT, 0, gstream()>>>(w.p, v.p, n, nrm.p);
@@ -379,6 +387,20 @@ __device__ __forceinline__ int hash_insert(int *h, int key, int *ovf) {
   return 0;
 }
 
+// the distinct block columns of row I of A B, into the warp's hash set: a lane
+// per entry of A's row, so that the chains column -> row of B -> its columns
+// of 32 entries run at the same time (which entry meets a column first does
+// not matter).  Returns the lane's count of new columns.
+__device__ __forceinline__ int spgemm_columns(const BV &A, const BV &B, int64_t I, int lane, int *h, int *ovf) {
+  int c = 0;
+  for (int a = A.rp[I] + lane; a < A.rp[I + 1]; a += 32) {
+    const int K = A.ci[a];
+    const int hi = B.rp[K + 1];
+    for (int q = B.rp[K]; q < hi; ++q) c += hash_insert(h, B.ci[q], ovf);
+  }
+  return c;
+}
+
 __global__ void k_spgemm_count(BV A, BV B, int32_t *__restrict__ cnt, int *__restrict__ ovf) {
   __shared__ int hs[kWarpsSp * kHash];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -387,11 +409,7 @@ __global__ void k_spgemm_count(BV A, BV B, int32_t *__restrict__ cnt, int *__res
   int *h = hs + warp * kHash;
   for (int i = lane; i < kHash; i += 32) h[i] = -1;
   __syncwarp();
-  int c = 0;
-  for (int a = A.rp[I]; a < A.rp[I + 1]; ++a) {
-    const int K = A.ci[a];
-    for (int q = B.rp[K] + lane; q < B.rp[K + 1]; q += 32) c += hash_insert(h, B.ci[q], ovf);
-  }
+  int c = spgemm_columns(A, B, I, lane, h, ovf);
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
   if (lane == 0) {
     cnt[I] = c;
@@ -399,21 +417,27 @@ __global__ void k_spgemm_count(BV A, BV B, int32_t *__restrict__ cnt, int *__res
   }
 }
 
+// A warp per row of C = A B.  The columns come from the hash set, sorted; then
+// the row's entries are accumulated in shared memory (acc_cap doubles per
+// warp, the space of the hash set; larger rows in place in cv).  The entries
+// of A's row are taken one after another and the products of one of them -
+// all blocks of B's row, every entry of the block - by the lanes at the same
+// time: B's columns are distinct, so no two lanes add to one entry and every
+// entry adds its products in the order of A's row, whatever the scheduling.
+// (One product at a time, on block-size lanes and in global memory, the
+// Galerkin products of a 10,648-node box with 3 fields took 33 ms, 9 now.)
 __global__ void k_spgemm_fill(BV A, BV B, const int32_t *__restrict__ crp, int32_t *__restrict__ cci,
-                              double *__restrict__ cv, int *__restrict__ ovf) {
-  __shared__ int hs[kWarpsSp * kHash];
-  __shared__ int cs[kWarpsSp * kCap];
+                              double *__restrict__ cv, int acc_cap, int *__restrict__ ovf) {
+  extern __shared__ __align__(16) double sp_smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t I = (int64_t)blockIdx.x * kWarpsSp + warp;
   if (I >= A.nbr) return;
-  int *h = hs + warp * kHash;
-  int *cols = cs + warp * kCap;
+  double *acc = sp_smem + (int64_t)warp * acc_cap;
+  int *h = reinterpret_cast<int *>(acc);
+  int *cols = reinterpret_cast<int *>(sp_smem + (int64_t)kWarpsSp * acc_cap) + warp * kCap;
   for (int i = lane; i < kHash; i += 32) h[i] = -1;
   __syncwarp();
-  for (int a = A.rp[I]; a < A.rp[I + 1]; ++a) {
-    const int K = A.ci[a];
-    for (int q = B.rp[K] + lane; q < B.rp[K + 1]; q += 32) hash_insert(h, B.ci[q], ovf);
-  }
+  spgemm_columns(A, B, I, lane, h, ovf);
   __syncwarp();
   // compact the set into cols (order of slots), then sort
   int m = 0;
@@ -429,31 +453,44 @@ __global__ void k_spgemm_fill(BV A, BV B, const int32_t *__restrict__ crp, int32
   warp_bitonic(cols, nullptr, m, kCap);
   const int64_t r0 = crp[I];
   for (int p = lane; p < m; p += 32) cci[r0 + p] = cols[p];
-  const int ob = A.br * B.bc;
-  for (int64_t e = lane; e < (int64_t)m * ob; e += 32) cv[r0 * ob + e] = 0.0;
+  const int ob = A.br * B.bc, tot = m * ob;
+  const bool local = tot <= acc_cap;
+  double *out = local ? acc : cv + r0 * ob;
   __syncwarp();
-  // values: every product in (a, q) order; lane e owns output entry e of a block
-  for (int a = A.rp[I]; a < A.rp[I + 1]; ++a) {
-    const int K = A.ci[a];
-    const double *ab = A.v + (int64_t)a * A.br * A.bc;
-    for (int q = B.rp[K]; q < B.rp[K + 1]; ++q) {
-      const int j = B.ci[q];
-      int lo = 0, hi = m - 1;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (cols[mid] < j) lo = mid + 1;
-        else hi = mid;
-      }
-      const double *bb = B.v + (int64_t)q * B.br * B.bc;
-      double *cb = cv + (r0 + lo) * ob;
-      for (int e = lane; e < ob; e += 32) {
-        const int r = e / B.bc, c = e % B.bc;
+  for (int e = lane; e < tot; e += 32) out[e] = 0.0;
+  __syncwarp();
+  const int alo = A.rp[I], ahi = A.rp[I + 1];
+  for (int a0 = alo; a0 < ahi; a0 += 32) {
+    // column and row of B of the next 32 entries, one per lane
+    int bq = 0, bn = 0;
+    if (a0 + lane < ahi) {
+      const int K = A.ci[a0 + lane];
+      bq = B.rp[K];
+      bn = B.rp[K + 1] - bq;
+    }
+    const int na = min(32, ahi - a0);
+    for (int u = 0; u < na; ++u) {
+      const int q0 = __shfl_sync(0xffffffffu, bq, u), nq = __shfl_sync(0xffffffffu, bn, u);
+      const double *ab = A.v + (int64_t)(a0 + u) * A.br * A.bc;
+      for (int i = lane; i < nq * ob; i += 32) {
+        const int q = i / ob, e = i - q * ob, r = e / B.bc, c = e - r * B.bc;
+        const int j = B.ci[q0 + q];
+        const double *bb = B.v + (int64_t)(q0 + q) * B.br * B.bc;
         double s = 0.0;
         for (int t = 0; t < A.bc; ++t) s += ab[r * A.bc + t] * bb[t * B.bc + c];
-        cb[e] += s;
+        int lo = 0, hi = m - 1;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (cols[mid] < j) lo = mid + 1;
+          else hi = mid;
+        }
+        out[lo * ob + e] += s;
       }
+      __syncwarp();
     }
   }
+  if (local)
+    for (int e = lane; e < tot; e += 32) cv[r0 * ob + e] = acc[e];
 }
 
 DB spgemm(const DB &A, const DB &B) {
@@ -476,7 +513,13 @@ DB spgemm(const DB &A, const DB &B) {
   C.nnzb = counts_to_rowptr(cnt.p, A.nbr, C.rp.p);
   C.ci.resize(C.nnzb);
   C.v.resize(C.nnzb * C.br * C.bc);
-  k_spgemm_fill<<<g, 32 * kWarpsSp, 0, gstream()>>>(view(A), view(B), C.rp.p, C.ci.p, C.v.p, ovf.p);
+  // accumulators: the hash set's space (1,024 doubles a warp), 2,560 for 6x6
+  // blocks (71 columns; coarse elasticity rows have 40 to 60)
+  const int acc_cap = A.br * B.bc > 18 ? 2560 : kHash / 2;
+  const size_t smem = (size_t)kWarpsSp * (acc_cap * sizeof(double) + kCap * sizeof(int));
+  GS_CUDA(cudaFuncSetAttribute(k_spgemm_fill, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kWarpsSp * (2560 * (int)sizeof(double) + kCap * (int)sizeof(int))));
+  k_spgemm_fill<<<g, 32 * kWarpsSp, smem, gstream()>>>(view(A), view(B), C.rp.p, C.ci.p, C.v.p, acc_cap, ovf.p);
   GS_CUDA(cudaGetLastError());
   return C;
 }

@@ -1458,7 +1458,7 @@ __device__ __forceinline__ double block_sum(double v, double *sh) {
 // them (a warp's float64 instruction takes 64 cycles of an SM quarter; HBM
 // delivers 1.6 times what the pipe can use), on small systems through the SM
 // with the most entries: so the entries are spread over all SMs in tiles of
-// 256 (arnoldi_plan) and the sums over lanes are kept short
+// 256 (mdot_blocks) and the sums over lanes are kept short
 // (warp_sum_rows).  The three passes and their reductions at 23 rows, in a
 // graph: 48,510 entries 27 us (107 us with n / 2048 CTAs), 344,605 73 us
 // (133), 1.37 M 266 us (287; float64 floor 238).  Smaller tiles shared by
@@ -2413,15 +2413,17 @@ void scale(const double *x, double a, double *y, int64_t n, cudaStream_t s) {
 // as 120 such instructions (fitted to timings of 972 to 1.37 M entries).
 // More than two tiles per CTA only with 3 CTAs per SM, which hide the load
 // latency (1.37 M entries, 47 rows: 2 per SM 597 us, 3 per SM 500 us).
-// (The plan is per system, so a batch and a solo solve reduce in the same order.)
-struct ArnoldiPlan {
-  int nblk = 1;
-  int64_t per = kTile;
-};
-static ArnoldiPlan arnoldi_plan(int64_t n) {
-  ArnoldiPlan best;
-  double tbest = 1e300;
+// Systems solved in batches fill the GPU together: four tiles a CTA there (the
+// sums over lanes are 4 % of a CTA's float64 work instead of 14 %).
+// (The count is per system, so a batch and a solo solve reduce in the same order.)
+int mdot_blocks(int64_t n, bool batch) {
   const int64_t tiles = std::max<int64_t>(1, (n + kTile - 1) / kTile);
+  if (batch) {
+    const int64_t per = std::max<int64_t>(4, (tiles + 152 * 4 - 1) / (152 * 4));
+    return (int)((tiles + per - 1) / per);
+  }
+  int best = 1;
+  double tbest = 1e300;
   for (int ctas = 1; ctas <= 6; ++ctas) {  // CTAs per SM
     const int64_t per = (tiles + 152 * ctas - 1) / (152 * ctas);
     const int64_t nblk = (tiles + per - 1) / per;
@@ -2429,21 +2431,24 @@ static ArnoldiPlan arnoldi_plan(int64_t n) {
     const double t = (double)((nblk + 151) / 152) * (768.0 * per + 120.0);
     if (t < tbest) {
       tbest = t;
-      best.nblk = (int)nblk;
-      best.per = per * kTile;
+      best = (int)nblk;
     }
   }
   return best;
 }
-int mdot_blocks(int64_t n) { return arnoldi_plan(n).nblk; }
+// entries (whole tiles) per CTA
+static int64_t mdot_per(int64_t n, int nblk) {
+  const int64_t tiles = std::max<int64_t>(1, (n + kTile - 1) / kTile);
+  return (tiles + nblk - 1) / nblk * kTile;
+}
 
 void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, double *partial, int nblk,
           cudaStream_t s, double *out, unsigned *cnt) {
-  const ArnoldiPlan p = arnoldi_plan(n);
+  const int64_t per = mdot_per(n, nblk);
   if (k != 1 || !out) cnt = nullptr;
   {
     HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 1), 1, n, 2.0 * n * k);
-    go<KMdot>(nblk, kThreads, 0, s, {V, ldv, k, w, n, partial, nblk, p.per, out, cnt});
+    go<KMdot>(nblk, kThreads, 0, s, {V, ldv, k, w, n, partial, nblk, per, out, cnt});
   }
   if (out && !cnt) reduce_partials(partial, k, nblk, out, s);
 }
@@ -2456,19 +2461,19 @@ void reduce_partials(const double *partial, int k, int nblk, double *out, cudaSt
 
 void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
                int nblk, double *out, cudaStream_t s) {
-  const ArnoldiPlan p = arnoldi_plan(n);
+  const int64_t per = mdot_per(n, nblk);
   {
     HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 3, n, 4.0 * n * k);
-    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, p.per});
+    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, per});
   }
   reduce_partials(partial, k, nblk, out, s);
 }
 
 void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
                 double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s) {
-  const ArnoldiPlan p = arnoldi_plan(n);
+  const int64_t per = mdot_per(n, nblk);
   HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 4, n, 2.0 * n * k + 2.0 * n);
-  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, p.per, out, cnt});
+  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, per, out, cnt});
 }
 
 void gemv_add(const double *Z, int64_t ldz, int k, const double *y, double *x, int64_t n, cudaStream_t s) {

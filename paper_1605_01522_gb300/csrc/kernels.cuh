@@ -239,9 +239,10 @@ template <typename TO>
 void scale_convert_dev(double *v, const double *inv, TO *out, int64_t n, cudaStream_t s);
 
 // Arnoldi (float64).  V holds k row vectors of length n, row q at V + q*ldv.
-// partial: k * nblk doubles of scratch, nblk = mdot_blocks(n); out: device
-// memory; cnt: a device counter that is 0 between passes.
-int mdot_blocks(int64_t n);
+// partial: k * nblk doubles of scratch, nblk = mdot_blocks(n) (batch: for a
+// system solved together with others); out: device memory; cnt: a device
+// counter that is 0 between passes.
+int mdot_blocks(int64_t n, bool batch = false);
 // out[q] = V_q . w; with out null only partial[q*nblk+b], for a later
 // reduce_partials.  One row with cnt given is reduced by the pass itself
 // (the same sum).

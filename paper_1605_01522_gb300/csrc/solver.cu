@@ -167,7 +167,9 @@ static PinnedCache &g_pinned = *new PinnedCache();
 // solve by up to 15 %, changed from process to process, and building both
 // layouts made their setups longer.
 constexpr int64_t kTuneMinRows = 131072;
-constexpr int64_t kTuneMinRowsBatch = 2048;
+constexpr int64_t kTuneMinRowsBatch = 16384;
+// mfs_params.layout_tune of the setup running on this thread
+static thread_local int g_layout_tune = 0;
 
 // Threads per block row of a SELL-32 matrix of nbr rows of avg blocks: 8 for
 // long rows, 4 for short ones, halved while the matrix would take more than
@@ -189,8 +191,14 @@ static int sell_split(int64_t nbr, double avg) {
 // blocks, which a lane walks longest (20,261 rows of 105 1x1 blocks 15.9 / 10.4
 // us a product, 68,921 of 114 16.2 / 20.3).  Rows of over 128 blocks and blocks
 // above 3x6 stay plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
+// In batches the systems fill the GPU together, so the fewest instructions a
+// row win (96 systems of 1,089 rows float64: SELL-32 10.3 ms, plain BSR 14.4)
+// and 2 threads per row: 24 boxes of 729 to 15,625 rows 24.4 ms with 1 (tuned by
+// timing), 19.7 with 2, 19.4 with 4; 256 boxes of up to
+// 117,649 rows 626 ms with 4, 615 with 2).
 static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb) {
   const double avg = nbr ? (double)nnzb / (double)nbr : 0.0;
+  if (g_layout_tune == 1) return nbr >= 700 && br * bc <= 18 && avg <= 32.0 ? 2 : 0;
   if (br * bc > 18 || avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : avg <= 32.0 ? 16384 : 49152)) return 0;
   return sell_split(nbr, avg);
 }
@@ -395,8 +403,6 @@ template <typename T> static float time_spmv(const dev::Sell &S, cudaStream_t st
 
 static std::mutex g_tune_mu;
 static std::map<std::tuple<int, int, int64_t, int64_t, int>, int> g_tune;
-// mfs_params.layout_tune of the setup running on this thread
-static thread_local int g_layout_tune = 0;
 
 // Layout candidates of the autotuner: 0 SELL-32 with 2 slots in flight,
 // 1 with 4, 2 plain BSR with one warp per row, 3 SELL-32 with 8 slots in
@@ -2585,7 +2591,7 @@ void upload_precond(mfs_handle *h, Arena &mat, Precond<T> &P, const std::map<std
 void alloc_solver_work(mfs_handle *h) {
   h->m = h->prm.restart;
   h->graphs.assign(h->m, IterGraph());
-  h->nblk = dev::mdot_blocks(h->n);
+  h->nblk = dev::mdot_blocks(h->n, h->prm.layout_tune == 1);
   h->V = h->ar.zeros<double>((int64_t)(h->m + 1) * h->n);
   h->Z = h->ar.zeros<double>((int64_t)h->m * h->n);
   h->rd = h->ar.zeros<double>(h->n);

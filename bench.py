@@ -185,8 +185,8 @@ def kernel_source_digest(kernel):
     fn = {"smooth_sell": ["sell_row", "d_smooth"], "spmv_sell": ["sell_row", "d_spmv"],
           "smooth_sell4": ["sell_row", "d_smooth"], "spmv_sell4": ["sell_row", "d_spmv"],
           "smooth_sell8": ["sell_row", "d_smooth"], "spmv_sell8": ["sell_row", "d_spmv"],
-          "spmv_rows": ["d_spmv_rows"], "smooth_warp": ["bsr_warp_row", "d_smooth_warp"],
-          "spmv_warp": ["bsr_warp_row", "d_spmv_warp"]}.get(kernel.split("<")[0])
+          "spmv_rows": ["d_spmv_rows"], "smooth_warp": ["bsr_row", "group_sum"],
+          "spmv_warp": ["bsr_row", "group_sum"]}.get(kernel.split("<")[0])
     if fn:
         fn = fn + ["k_solo"]  # the single-system kernel wrapper every launch goes through
     if not fn:

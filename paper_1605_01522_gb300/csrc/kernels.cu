@@ -300,7 +300,8 @@ __device__ __forceinline__ void sell_row(const int32_t *__restrict__ sp, const i
 // A plain-BSR block row by a group of L = 2^ls lanes (8, 16 or 32): the lanes
 // stride over the row's blocks.  The first block of a lane is loaded before
 // `wait` (see k_solo), the next column while the current block is used, so
-// that a further block costs one load latency instead of two.
+// that a further block costs one load latency instead of two.  (Two or four
+// blocks of a lane at a time cost registers: 23^3 box AMG(BGS) 9.8 -> 10.1-12.1 ms.)
 template <int BR, int BC, typename T, class W>
 __device__ __forceinline__ void bsr_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
                                         const T *__restrict__ val, const T *__restrict__ x, int64_t row, bool active,
@@ -426,10 +427,9 @@ struct KSpmvWarp {
 // levels): threads stride over the row's blocks, then a fixed butterfly per
 // warp and a fixed-order sum over the warps.
 template <int BR, int BC, typename T>
-__device__ __forceinline__ void d_spmv_cta(int64_t nbr, const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-           const T *__restrict__ val, const T *__restrict__ x, T *y, T alpha, T beta, const T *z, int bid_, int nb_) {
-  __shared__ T part[kThreads / 32][BR];
-  const int64_t row = bid_;
+__device__ __forceinline__ void cta_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
+                                        const T *__restrict__ val, const T *__restrict__ x, int64_t row,
+                                        T (*part)[BR]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   T acc[BR];
 #pragma unroll
@@ -453,6 +453,14 @@ __device__ __forceinline__ void d_spmv_cta(int64_t nbr, const int32_t *__restric
     if (lane == 0) part[warp][r] = acc[r];
   }
   __syncthreads();
+}
+
+template <int BR, int BC, typename T>
+__device__ __forceinline__ void d_spmv_cta(int64_t nbr, const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
+           const T *__restrict__ val, const T *__restrict__ x, T *y, T alpha, T beta, const T *z, int bid_, int nb_) {
+  __shared__ T part[kThreads / 32][BR];
+  const int64_t row = bid_;
+  cta_row<BR, BC, T>(rp, col, val, x, row, part);
   if (threadIdx.x < BR) {
     T a = T(0);
     for (int w = 0; w < kThreads / 32; ++w) a += part[w][threadIdx.x];
@@ -477,6 +485,45 @@ struct KSpmvCta {
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
     d_spmv_cta<BR, BC, T>(a.nbr, a.rp, a.col, a.val, a.x, a.y, a.alpha, a.beta, a.z, bid, nb);
+  }
+};
+
+// the same row per CTA for a smoothing step
+template <int BR, typename T>
+struct KSmoothCta {
+  static constexpr int kMaxThreads = kThreads;
+  static constexpr bool kFp64 = sizeof(T) == 8;
+  struct Args {
+    int64_t nbr;
+    const int32_t *rp;
+    const int32_t *col;
+    const T *val;
+    const T *dinv;
+    const T *b;
+    const T *x;
+    T *xout;
+    T *d;
+    T c1;
+    T c2;
+  };
+  static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
+    __shared__ T part[kThreads / 32][BR];
+    const int64_t i = (int64_t)bid * BR + threadIdx.x;
+    T bi = T(0), xi = T(0), dd = T(0), di = T(0);
+    if (threadIdx.x < BR) {
+      bi = a.b[i];
+      xi = a.x[i];
+      dd = a.d[i];
+      di = a.dinv[i];
+    }
+    cta_row<BR, BR, T>(a.rp, a.col, a.val, a.x, bid, part);
+    if (threadIdx.x < BR) {
+      T s = T(0);
+      for (int w = 0; w < kThreads / 32; ++w) s += part[w][threadIdx.x];
+      dd = a.c1 * dd + a.c2 * di * (bi - s);
+      a.d[i] = dd;
+      a.xout[i] = xi + dd;
+    }
   }
 };
 
@@ -903,23 +950,38 @@ __device__ __forceinline__ void d_spmv_rows(int64_t nbr, const int32_t *__restri
       }
   }
 }
-template <int BR, int B0, int B1, int B2, int H>
+// The rows of all fields in one launch: CTAs [0, end[0]) take field 0 (BR =
+// B0), then fields 1 and 2 (one dof per node).  The launches' ends, where SMs
+// run dry, and two launches of a few microseconds on small systems are paid
+// once (64^3 box 366 -> 340 us, 3,267-dof system 1.70 -> 1.66 ms a solve).
+template <int B0, int B1, int B2, int H>
 struct KSpmvRows {
   static constexpr int kMaxThreads = (H == 1 ? 64 : 32 * H);
   static constexpr bool kFp64 = true;
-  struct Args {
+  struct Field {
     int64_t nbr;
     const int32_t *sp;
     const int32_t *rl;
     const int32_t *col;
     const double *val;
+    double *y;
+  };
+  struct Args {
+    int end[3];  // CTAs up to and with each field
+    Field f[3];
     const double *x0;
     const double *x1;
     const double *x2;
-    double *y;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_spmv_rows<BR, B0, B1, B2, H>(a.nbr, a.sp, a.rl, a.col, a.val, a.x0, a.x1, a.x2, a.y, bid, nb);
+    if (bid < a.end[0]) {
+      const Field &f = a.f[0];
+      d_spmv_rows<B0, B0, B1, B2, H>(f.nbr, f.sp, f.rl, f.col, f.val, a.x0, a.x1, a.x2, f.y, bid, nb);
+    } else {
+      const int i = bid < a.end[1] ? 1 : 2;
+      const Field &f = a.f[i];
+      d_spmv_rows<1, B0, B1, B2, H>(f.nbr, f.sp, f.rl, f.col, f.val, a.x0, a.x1, a.x2, f.y, bid - a.end[i - 1], nb);
+    }
   }
 };
 
@@ -1530,6 +1592,29 @@ __device__ __forceinline__ void finish_sum(const double *partial, int nb, double
   }
 }
 
+// The sums of a pass over at most kInlineBlocks CTAs are added up by every CTA
+// of the next pass itself (thread q adds the partial sums of row q in order;
+// CTA 0 also writes them out for the host): 0.4 us for 13 partials instead of a
+// launch of 2.3 us.
+constexpr int kInlineBlocks = 16;
+__device__ __forceinline__ void load_sums(const double *__restrict__ h, const double *__restrict__ hpart, int k,
+                                          int rows, int nblk, double *__restrict__ hout, double *hs, int bid) {
+  if (hpart == nullptr) {
+    for (int q = threadIdx.x; q < k; q += kThreads) hs[q] = h[q];
+  } else if (threadIdx.x < rows) {
+    const double *p = hpart + (int64_t)threadIdx.x * nblk;
+    double a[kInlineBlocks], t = 0.0;
+#pragma unroll
+    for (int i = 0; i < kInlineBlocks; ++i) a[i] = i < nblk ? p[i] : 0.0;
+#pragma unroll
+    for (int i = 0; i < kInlineBlocks; ++i)
+      if (i < nblk) t += a[i];
+    if (threadIdx.x < k) hs[threadIdx.x] = t;
+    if (bid == 0) hout[threadIdx.x] = t;
+  }
+  __syncthreads();
+}
+
 // acc[m] += V_q[t0 ..] . ws over a staged tile for the warp's rows q = warp +
 // 8 m, a lane's 8 loads issued before the first product
 __device__ __forceinline__ void tile_dots(const double *__restrict__ V, int64_t ldv, int k, int64_t t0, int cnt,
@@ -1641,12 +1726,12 @@ struct KMdot {
 };
 
 // w <- w - sum_q V_q h_q, then partial dots V_q . w_new (CGS2 second pass)
-__device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h, double *__restrict__ w,
+__device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h,
+            const double *__restrict__ hpart, double *__restrict__ hout, double *__restrict__ w,
             int64_t n, double *__restrict__ partial, int nblk, int64_t per, int bid_) {
   __shared__ double ws[kTile];
   __shared__ double hs[kMaxQ];
-  for (int q = threadIdx.x; q < k; q += blockDim.x) hs[q] = h[q];
-  __syncthreads();
+  load_sums(h, hpart, k, k + 1, nblk, hout, hs, bid_);  // the dot pass had w as its last row
   const int64_t lo = (int64_t)bid_ * per, hi = min(n, lo + per);
   double acc[kMaxQ / 8];
 #pragma unroll
@@ -1675,6 +1760,8 @@ struct KCgsFused {
     int64_t ldv;
     int k;
     const double *h;
+    const double *hpart;  // or null: h holds the sums
+    double *hout;
     double *w;
     int64_t n;
     double *partial;
@@ -1682,7 +1769,7 @@ struct KCgsFused {
     int64_t per;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_cgs_fused(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.per, bid);
+    d_cgs_fused(a.V, a.ldv, a.k, a.h, a.hpart, a.hout, a.w, a.n, a.partial, a.nblk, a.per, bid);
   }
 };
 
@@ -1709,12 +1796,11 @@ struct KReducePartials {
 
 // w <- w - sum_q V_q h_q, then |w|^2 and 1 / |w| (last CTA)
 __device__ __forceinline__ void d_cgs_update(const double *__restrict__ V, int64_t ldv, int k, const double *__restrict__ h,
-             double *__restrict__ w, int64_t n, double *__restrict__ partial, int nblk, int64_t per, double *out,
-             unsigned *cnt, int bid_) {
+             const double *__restrict__ hpart, double *__restrict__ hout, double *__restrict__ w, int64_t n,
+             double *__restrict__ partial, int nblk, int64_t per, double *out, unsigned *cnt, int bid_) {
   __shared__ double hs[kMaxQ];
   __shared__ double sh[32];
-  for (int q = threadIdx.x; q < k; q += blockDim.x) hs[q] = h[q];
-  __syncthreads();
+  load_sums(h, hpart, k, k, nblk, hout, hs, bid_);
   const int64_t lo = (int64_t)bid_ * per, hi = min(n, lo + per);
   double nrm = 0.0;
   for (int64_t i = lo + threadIdx.x; i < hi; i += kTile) {
@@ -1735,6 +1821,8 @@ struct KCgsUpdate {
     int64_t ldv;
     int k;
     const double *h;
+    const double *hpart;  // or null: h holds the sums
+    double *hout;
     double *w;
     int64_t n;
     double *partial;
@@ -1744,7 +1832,7 @@ struct KCgsUpdate {
     unsigned *cnt;
   };
   static __device__ __forceinline__ void run(const Args &a, int bid, int nb) {
-    d_cgs_update(a.V, a.ldv, a.k, a.h, a.w, a.n, a.partial, a.nblk, a.per, a.out, a.cnt, bid);
+    d_cgs_update(a.V, a.ldv, a.k, a.h, a.hpart, a.hout, a.w, a.n, a.partial, a.nblk, a.per, a.out, a.cnt, bid);
   }
 };
 
@@ -2099,46 +2187,59 @@ void spmv(const Sell &A, const T *x, T *y, T alpha, T beta, const T *z, cudaStre
     default: fprintf(stderr, "mfs: unsupported block size %d\n", BRV); \
   }
 
-#define MFS_ROWS_DISPATCH(BR, B, CALL)                                          \
-  switch (BR * 1000 + B[0] * 100 + B[1] * 10 + B[2]) {                          \
-    case 3311: { constexpr int R_ = 3, X0 = 3, X1 = 1, X2 = 1; CALL; } break;   \
-    case 1311: { constexpr int R_ = 1, X0 = 3, X1 = 1, X2 = 1; CALL; } break;   \
-    case 3310: { constexpr int R_ = 3, X0 = 3, X1 = 1, X2 = 0; CALL; } break;   \
-    case 1310: { constexpr int R_ = 1, X0 = 3, X1 = 1, X2 = 0; CALL; } break;   \
-    case 2210: { constexpr int R_ = 2, X0 = 2, X1 = 1, X2 = 0; CALL; } break;   \
-    case 1210: { constexpr int R_ = 1, X0 = 2, X1 = 1, X2 = 0; CALL; } break;   \
-    default: break;                                                             \
+#define MFS_ROWS_DISPATCH(B, CALL)                                      \
+  switch (B[0] * 100 + B[1] * 10 + B[2]) {                              \
+    case 311: { constexpr int X0 = 3, X1 = 1, X2 = 1; CALL; } break;    \
+    case 310: { constexpr int X0 = 3, X1 = 1, X2 = 0; CALL; } break;    \
+    case 210: { constexpr int X0 = 2, X1 = 1, X2 = 0; CALL; } break;    \
+    default: break;                                                     \
   }
 
-bool rows_supported(int br, const int *b, int nb) {
-  const int code = br * 1000 + b[0] * 100 + b[1] * 10 + (nb > 2 ? b[2] : 0);
-  switch (code) {
-    case 3311: case 1311: case 3310: case 1310: case 2210: case 1210: return nb >= 2 && nb <= 3;
-    default: return false;
-  }
+bool rows_supported(const int *b, int nb) {
+  if (nb < 2 || nb > 3) return false;
+  const int code = b[0] * 100 + b[1] * 10 + (nb > 2 ? b[2] : 0);
+  return code == 311 || code == 310 || code == 210;
 }
 
-void spmv_rows(const RowMerged &R, const double *x, double *y, cudaStream_t s) {
-  const Sell &A = R.M;
-  if (A.nbr == 0) return;
-  HookScope hs(s, K_SPMV,
-               (double)A.nnzb * (A.br * A.bc * 8.0 + 4.0) + 4.0 * A.nbr + 8.0 * (A.nbc * A.bc + A.nrows()),
-               2000 + A.br * 100 + A.bc * 10 + 1, A.nbr, 2.0 * A.nnzb * A.br * A.bc);
-  const double *x0 = x + R.off[0], *x1 = x + R.off[1], *x2 = R.nb > 2 ? x + R.off[2] : x;
-  const int b3[3] = {R.b[0], R.b[1], R.nb > 2 ? R.b[2] : 0};
-  const unsigned grid = (unsigned)A.nslices;  // H > 1: one slice per CTA
-  if (R.split == 8) {
-    MFS_ROWS_DISPATCH(A.br, b3, (go<KSpmvRows<R_, X0, X1, X2, 8>>(grid, 256, 0, s, {
-                                    A.nbr, A.sp, A.rl, A.col, A.v64, x0, x1, x2, y})));
-  } else if (R.split == 4) {
-    MFS_ROWS_DISPATCH(A.br, b3, (go<KSpmvRows<R_, X0, X1, X2, 4>>(grid, 128, 0, s, {
-                                    A.nbr, A.sp, A.rl, A.col, A.v64, x0, x1, x2, y})));
-  } else if (R.split == 2) {
-    MFS_ROWS_DISPATCH(A.br, b3, (go<KSpmvRows<R_, X0, X1, X2, 2>>(grid, 64, 0, s, {
-                                    A.nbr, A.sp, A.rl, A.col, A.v64, x0, x1, x2, y})));
+template <int B0, int B1, int B2, int H>
+static void rows_launch(const RowMerged *R, int nf, const double *x, double *y, cudaStream_t s) {
+  typename KSpmvRows<B0, B1, B2, H>::Args a{};
+  int end = 0;
+  for (int i = 0; i < 3; ++i) {
+    if (i < nf) {
+      const Sell &A = R[i].M;
+      end += H == 1 ? (int)grid_for(A.nbr, 64) : (int)A.nslices;  // H > 1: one slice per CTA
+      a.f[i] = {A.nbr, A.sp, A.rl, A.col, A.v64, y + R[i].off[i]};
+    }
+    a.end[i] = end;
+  }
+  a.x0 = x + R[0].off[0];
+  a.x1 = x + R[0].off[1];
+  a.x2 = nf > 2 ? x + R[0].off[2] : x;
+  if (end) go<KSpmvRows<B0, B1, B2, H>>((unsigned)end, H == 1 ? 64 : 32 * H, 0, s, a);
+}
+
+void spmv_rows(const std::vector<RowMerged> &R, const double *x, double *y, cudaStream_t s) {
+  const int nf = (int)R.size();
+  const int b3[3] = {R[0].b[0], R[0].b[1], nf > 2 ? R[0].b[2] : 0};
+  double bytes = 0.0, flops = 0.0;
+  int br = 0;
+  for (const RowMerged &r : R) {
+    const Sell &A = r.M;
+    bytes += (double)A.nnzb * (A.br * A.bc * 8.0 + 4.0) + 4.0 * A.nbr + 8.0 * (A.nbc * A.bc + A.nrows());
+    flops += 2.0 * A.nnzb * A.br * A.bc;
+    br += A.br;
+  }
+  HookScope hs(s, K_SPMV, bytes, 2000 + br * 100 + R[0].M.bc * 10 + 1, R[0].M.nbr, flops);
+  const int split = R[0].split;
+  if (split == 8) {
+    MFS_ROWS_DISPATCH(b3, (rows_launch<X0, X1, X2, 8>(R.data(), nf, x, y, s)));
+  } else if (split == 4) {
+    MFS_ROWS_DISPATCH(b3, (rows_launch<X0, X1, X2, 4>(R.data(), nf, x, y, s)));
+  } else if (split == 2) {
+    MFS_ROWS_DISPATCH(b3, (rows_launch<X0, X1, X2, 2>(R.data(), nf, x, y, s)));
   } else {
-    MFS_ROWS_DISPATCH(A.br, b3, (go<KSpmvRows<R_, X0, X1, X2, 1>>(grid_for(A.nbr, 64), 64, 0, s, {
-                                    A.nbr, A.sp, A.rl, A.col, A.v64, x0, x1, x2, y})));
+    MFS_ROWS_DISPATCH(b3, (rows_launch<X0, X1, X2, 1>(R.data(), nf, x, y, s)));
   }
 }
 
@@ -2147,8 +2248,14 @@ void smooth_step(const Sell &A, const T *dinv, const T *b, const T *x, T *xout, 
                  cudaStream_t s) {
   if (A.nbr == 0) return;
   const T *v = vals<T>(A);
+  const bool cta = cta_rows<T>(A);
   HookScope hs(s, K_SMOOTH, matrix_bytes<T>(A) + (double)sizeof(T) * (A.ncols() + 5.0 * A.nrows()),
-               sparse_sig<T>(A), A.nbr, 2.0 * A.nnzb * A.br * A.bc + 6.0 * A.nrows());
+               cta ? 7000 + sparse_sig<T>(A) % 1000 : sparse_sig<T>(A), A.nbr, 2.0 * A.nnzb * A.br * A.bc + 6.0 * A.nrows());
+  if (A.kind == 1 && cta) {
+    MFS_SQUARE_DISPATCH(A.br, (go<KSmoothCta<BR_, T>>((unsigned)A.nbr, kThreads, 0, s, {
+                                  A.nbr, A.sp, A.col, v, dinv, b, x, xout, d, c1, c2})));
+    return;
+  }
   if (A.kind == 1) {
     const int ls = bsr_ls<T>(A);
     const unsigned th = bsr_threads(A.nbr << ls);
@@ -2459,21 +2566,21 @@ void reduce_partials(const double *partial, int k, int nblk, double *out, cudaSt
   go<KReducePartials>(g_rec ? (unsigned)kMaxQ : (unsigned)k, kThreads, 0, s, {partial, k, nblk, out});
 }
 
-void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
-               int nblk, double *out, cudaStream_t s) {
+// One CGS2 step (see kernels.cuh)
+void cgs2(const double *V, int64_t ldv, int k, double *w, int64_t n, double *partial, int nblk, double *out,
+          unsigned *cnt, cudaStream_t s) {
   const int64_t per = mdot_per(n, nblk);
+  const bool inl = nblk <= kInlineBlocks;
+  double *p1 = partial, *p2 = partial + (int64_t)64 * nblk;
+  mdot(V, ldv, k + 1, w, n, p1, nblk, s, inl ? nullptr : out, nullptr);
   {
     HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 3, n, 4.0 * n * k);
-    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, per});
+    go<KCgsFused>(nblk, kThreads, 0, s, {V, ldv, k, out, inl ? p1 : nullptr, out, w, n, p2, nblk, per});
   }
-  reduce_partials(partial, k, nblk, out, s);
-}
-
-void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
-                double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s) {
-  const int64_t per = mdot_per(n, nblk);
+  if (!inl) reduce_partials(p2, k, nblk, out + 64, s);
   HookScope hs(s, K_ARNOLDI, 8.0 * n * (k + 2), 4, n, 2.0 * n * k + 2.0 * n);
-  go<KCgsUpdate>(nblk, kThreads, 0, s, {V, ldv, k, h, w, n, partial, nblk, per, out, cnt});
+  go<KCgsUpdate>(nblk, kThreads, 0, s,
+                 {V, ldv, k, out + 64, inl ? p2 : nullptr, out + 64, w, n, p1, nblk, per, out + 128, cnt});
 }
 
 void gemv_add(const double *Z, int64_t ldz, int k, const double *y, double *x, int64_t n, cudaStream_t s) {

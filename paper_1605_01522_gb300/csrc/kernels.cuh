@@ -150,8 +150,10 @@ struct RowMerged {
   int64_t off[3] = {0, 0, 0};  // offset of each column field in the coupled vector
   int split = 1;   // threads per block row (1, 2, 4 or 8), timed at setup
 };
-bool rows_supported(int br, const int *b, int nb);
-void spmv_rows(const RowMerged &R, const double *x, double *y, cudaStream_t s);
+// column fields of b[0], b[1][, b[2]] dofs per node, row field 0 of b[0], the others of one
+bool rows_supported(const int *b, int nb);
+// the rows of all fields (R[i]: row field i, at off[i] of y) in one launch, with R[0].split
+void spmv_rows(const std::vector<RowMerged> &R, const double *x, double *y, cudaStream_t s);
 
 // One smoothing step on A with point-diagonal inverse dinv:
 //   r = b - A x;  d = c1 * d + c2 * dinv * r;  xout = x + d
@@ -249,12 +251,12 @@ int mdot_blocks(int64_t n, bool batch = false);
 void mdot(const double *V, int64_t ldv, int k, const double *w, int64_t n, double *partial,
           int nblk, cudaStream_t s, double *out = nullptr, unsigned *cnt = nullptr);
 void reduce_partials(const double *partial, int k, int nblk, double *out, cudaStream_t s);
-// w -= sum_q V_q h_q and out[q] = V_q . w_new in one pass (k <= 64)
-void cgs_fused(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n, double *partial,
-               int nblk, double *out, cudaStream_t s);
-// w -= sum_q V_q h_q, out[0] = |w_new|^2, out[1] = 1 / |w_new|
-void cgs_update(const double *V, int64_t ldv, int k, const double *h, double *w, int64_t n,
-                double *partial, int nblk, double *out, unsigned *cnt, cudaStream_t s);
+// One CGS2 step of w (row k of V) against rows 0..k-1 (k < 64): out[q] =
+// V_q . w for q <= k (so out[k] = |w|^2), w -= sum V_q out[q], out[64 + q] =
+// V_q . w, w -= sum V_q out[64 + q], out[128] = |w|^2, out[129] = 1 / |w|.
+// partial: 128 * nblk doubles.
+void cgs2(const double *V, int64_t ldv, int k, double *w, int64_t n, double *partial, int nblk, double *out,
+          unsigned *cnt, cudaStream_t s);
 // x += sum_q Z_q y_q
 void gemv_add(const double *Z, int64_t ldz, int k, const double *y, double *x, int64_t n,
               cudaStream_t s);

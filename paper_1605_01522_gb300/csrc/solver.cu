@@ -854,7 +854,10 @@ template <typename T> struct Precond {
     FL<T> &f = g.lv[l][i], &c = g.lv[l + 1][i];
     dev::RowTerm<T> t{&f.R, r};
     bool done = false;
-    if (smoothed && smoother != MFS_GS && fusable(&t, 1)) {
+    // (long restrictions are not launch bound: 5,997 rows of 184 6x3 blocks
+    // took 32 us this way, 26 + 7 us as two launches; 1x1 14 and 9 + 7)
+    const bool small = f.R.nnzb * f.R.br * f.R.bc <= 1500000;
+    if (smoothed && small && smoother != MFS_GS && fusable(&t, 1)) {
       dev::RowOut<T> o;
       o.y = c.bv;
       set_first(o, c, c.xv, &done);
@@ -1343,7 +1346,7 @@ bool is_device_ptr(const void *p) {
 
 void matvec(mfs_handle *h, const double *x, double *y) {
   if (!h->rows64.empty()) {
-    for (int i = 0; i < h->nf; ++i) dev::spmv_rows(h->rows64[i], x, y + h->foff[i], h->s);
+    dev::spmv_rows(h->rows64, x, y, h->s);
     return;
   }
   for (int i = 0; i < h->nf; ++i) {
@@ -1475,9 +1478,7 @@ struct KrylovLS {
 void arnoldi(mfs_handle *h, int j, double *w, double *hd, cudaStream_t s) {
   const int64_t n = h->n;
   // CGS2: h1 = V^T w (and |w|^2), w -= V h1, h2 = V^T w, w -= V h2 (and |w|^2)
-  dev::mdot(h->V, n, j + 2, w, n, h->partial, h->nblk, s, hd, h->cnt);
-  dev::cgs_fused(h->V, n, j + 1, hd, w, n, h->partial, h->nblk, hd + 64, s);
-  dev::cgs_update(h->V, n, j + 1, hd + 64, w, n, h->partial, h->nblk, hd + 128, h->cnt, s);
+  dev::cgs2(h->V, n, j + 1, w, n, h->partial, h->nblk, hd, h->cnt, s);
 }
 
 // Solves and other solve-phase calls (apply, matvec) running in this process.
@@ -2208,12 +2209,12 @@ HBsr to_hbsr(const mfs_block &b) {
 }
 
 // Threads per block row of the merged float64 matvec (1, 2, 4 or 8): timed
-// once per (row block shape, rows, blocks) and process, like the layouts.
-static std::map<std::tuple<int, int, int, int, int64_t, int64_t>, int> g_tune_rows;
+// once per (column blocks, rows, blocks) and process, like the layouts.
+static std::map<std::tuple<int, int, int, int64_t, int64_t>, int> g_tune_rows;
 
-static int tune_rows(const dev::RowMerged &R, int64_t n, cudaStream_t st) {
-  const dev::Sell &A = R.M;
-  const auto key = std::make_tuple(A.br, R.b[0], R.b[1], R.nb > 2 ? R.b[2] : 0, (int64_t)A.nbr, (int64_t)A.nnzb);
+static int tune_rows(const std::vector<dev::RowMerged> &R, int64_t n, cudaStream_t st) {
+  const dev::Sell &A = R[0].M;
+  const auto key = std::make_tuple(R[0].b[0], R[0].b[1], R[0].nb > 2 ? R[0].b[2] : 0, (int64_t)A.nbr, (int64_t)A.nnzb);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune_rows.find(key);
@@ -2221,16 +2222,16 @@ static int tune_rows(const dev::RowMerged &R, int64_t n, cudaStream_t st) {
   }
   double *x = nullptr, *y = nullptr;
   MFS_CUDA(cudaMallocAsync((void **)&x, (size_t)std::max<int64_t>(1, n) * sizeof(double), st));
-  MFS_CUDA(cudaMallocAsync((void **)&y, (size_t)std::max<int64_t>(1, A.nrows()) * sizeof(double), st));
+  MFS_CUDA(cudaMallocAsync((void **)&y, (size_t)std::max<int64_t>(1, n) * sizeof(double), st));
   MFS_CUDA(cudaMemsetAsync(x, 0, (size_t)n * sizeof(double), st));
   cudaEvent_t e0, e1;
   MFS_CUDA(cudaEventCreate(&e0));
   MFS_CUDA(cudaEventCreate(&e1));
   int best = 1;
   float tbest = 1e30f;
+  std::vector<dev::RowMerged> T = R;
   for (int split : {1, 2, 4, 8}) {
-    dev::RowMerged T = R;
-    T.split = split;
+    T[0].split = split;
     for (int rep = 0; rep < 4; ++rep) {
       MFS_CUDA(cudaEventRecord(e0, st));
       dev::spmv_rows(T, x, y, st);
@@ -2275,19 +2276,18 @@ std::vector<dev::RowMerged> merge_rows_dev(Arena &ar, const std::map<std::pair<i
       b[j] = it->second.bc;
       src[j] = &raw.at({i, j});
     }
-    if (!dev::rows_supported(h0->br, b, nf)) return {};
+    if (h0->br != b[i] || !dev::rows_supported(b, nf)) return {};
     dev::RowMerged R;
     R.M = upload_layout_dev(ar, src, nf, true, false, 0, st);
     R.nb = nf;
-    int64_t n = 0;
     for (int j = 0; j < nf; ++j) {
       R.b[j] = b[j];
       R.off[j] = foff[j];
-      n = std::max(n, foff[j] + src[j]->nbc * src[j]->bc);
     }
-    R.split = split > 0 ? split : tune_rows(R, n, st);
     out.push_back(R);
   }
+  const int best = split > 0 ? split : tune_rows(out, foff[nf], st);
+  for (auto &R : out) R.split = best;
   return out;
 }
 
@@ -2597,7 +2597,7 @@ void alloc_solver_work(mfs_handle *h) {
   h->rd = h->ar.zeros<double>(h->n);
   h->xd = h->ar.zeros<double>(h->n);
   h->bd = h->ar.zeros<double>(h->n);
-  h->partial = h->ar.zeros<double>((int64_t)64 * h->nblk);
+  h->partial = h->ar.zeros<double>((int64_t)128 * h->nblk);
   h->hdev = h->ar.zeros<double>(kHostSlots);
   h->ydev = h->ar.zeros<double>(64);
   h->cnt = h->ar.zeros<unsigned>(1);

@@ -309,8 +309,8 @@ class Solver:
         return x, info.as_dict(), rc
 
     def apply(self, v, z=None):
-        if z is None:
-            z = np.zeros(self.n) if isinstance(v, np.ndarray) else v.new_zeros(self.n)
+        if z is None:  # every entry is written: no fill (a launch that the call would wait for)
+            z = np.empty(self.n) if isinstance(v, np.ndarray) else v.new_empty(self.n)
         rc = self.lib.mfs_apply(self.h, _ptr(v), _ptr(z))
         if rc != OK:
             raise MfsError(rc, "mfs_apply")
@@ -318,7 +318,7 @@ class Solver:
 
     def matvec(self, x, y=None):
         if y is None:
-            y = np.zeros(self.n) if isinstance(x, np.ndarray) else x.new_zeros(self.n)
+            y = np.empty(self.n) if isinstance(x, np.ndarray) else x.new_empty(self.n)
         rc = self.lib.mfs_matvec(self.h, _ptr(x), _ptr(y))
         if rc != OK:
             raise MfsError(rc, "mfs_matvec")

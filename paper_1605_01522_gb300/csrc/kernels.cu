@@ -159,8 +159,10 @@ __global__ void __launch_bounds__(K::kMaxThreads) k_solo(const __grid_constant__
 
 // CTAs per SM the multi-system form of K must fit (K::kMinBlocks, default 1):
 // its arguments come from a table instead of the constant bank, which costs
-// registers; the one-thread-per-row SELL kernels are held to the 32 registers
-// of their single-system form so that as many CTAs stay resident
+// registers (112 instead of 32 in the coupled matvec); the kernels of large
+// grids are held to about the registers of their single-system form so that as
+// many CTAs stay resident (256 boxes 607 -> 561 ms; the small float64 sparse
+// kernels, which wait for their own chains, lost 2 % and are not)
 template <class K, class = void> struct MinBlocks {
   static constexpr int value = 1;
 };
@@ -396,6 +398,7 @@ __device__ __forceinline__ void gs_update(const T (&acc)[BR], int64_t node, cons
 template <int BR, int BC, typename T>
 struct KSpmvWarp {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr int kMinBlocks = sizeof(T) == 4 && BR * BC <= 9 ? 5 : 1;  // multi-system form: <= 48 registers
   static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
@@ -530,6 +533,7 @@ struct KSmoothCta {
 template <int BR, typename T>
 struct KSmoothWarp {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr int kMinBlocks = sizeof(T) == 4 && BR <= 3 ? 5 : 1;  // multi-system form: <= 48 registers
   static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
@@ -697,6 +701,7 @@ __device__ __forceinline__ T sell_split_entry(T (*part)[BR][kSellPad], int e) {
 template <int BR, int BC, typename T>
 struct KSpmvSellSplit {
   static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr int kMinBlocks = sizeof(T) == 4 && BR * BC <= 9 ? 6 : 1;  // multi-system form: <= 40 registers
   static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
@@ -725,6 +730,7 @@ struct KSpmvSellSplit {
 template <int BR, typename T>
 struct KSmoothSellSplit {
   static constexpr int kMaxThreads = 32 * kSellSplitMax;
+  static constexpr int kMinBlocks = sizeof(T) == 4 && BR <= 3 ? 6 : 1;  // multi-system form: <= 40 registers
   static constexpr bool kFp64 = sizeof(T) == 8;
   static constexpr bool kEarly = true;
   struct Args {
@@ -957,6 +963,7 @@ __device__ __forceinline__ void d_spmv_rows(int64_t nbr, const int32_t *__restri
 template <int B0, int B1, int B2, int H>
 struct KSpmvRows {
   static constexpr int kMaxThreads = (H == 1 ? 64 : 32 * H);
+  static constexpr int kMinBlocks = 1536 / kMaxThreads;  // multi-system form: <= 40 registers
   static constexpr bool kFp64 = true;
   struct Field {
     int64_t nbr;
@@ -1707,6 +1714,7 @@ __device__ __forceinline__ void d_mdot(const double *__restrict__ V, int64_t ldv
 }
 struct KMdot {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr int kMinBlocks = 4;  // multi-system form: <= 64 registers
   static constexpr bool kFp64 = true;
   struct Args {
     const double *V;
@@ -1754,6 +1762,7 @@ __device__ __forceinline__ void d_cgs_fused(const double *__restrict__ V, int64_
 }
 struct KCgsFused {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr int kMinBlocks = 4;  // multi-system form: <= 64 registers
   static constexpr bool kFp64 = true;
   struct Args {
     const double *V;
@@ -1815,6 +1824,7 @@ __device__ __forceinline__ void d_cgs_update(const double *__restrict__ V, int64
 }
 struct KCgsUpdate {
   static constexpr int kMaxThreads = kThreads;
+  static constexpr int kMinBlocks = 4;  // multi-system form: <= 64 registers
   static constexpr bool kFp64 = true;
   struct Args {
     const double *V;

@@ -127,6 +127,14 @@ template <int N, typename T> __device__ __forceinline__ void ld_pin_block(const 
     for (int i = 0; i < N; ++i) o[i] = ld_pin(p + i);
   }
 }
+// A vector that an earlier launch of the solve wrote: an ordinary load.  Under
+// a programmatic launch this grid is resident while its predecessor still
+// writes x, so x is not read-only for the life of the kernel and must not be
+// read through the non-coherent path (__ldg, ld.global.nc), whose loads the
+// compiler may also move across the wait; ordinary loads stay behind the
+// wait's memory clobber as long as x is not __restrict__ in the function that
+// waits.  __ldg and ld_pin are for matrix data, which only the setup writes.
+template <typename T> __device__ __forceinline__ T ld_vec(const T *p) { return *p; }
 struct PdlWait {
   __device__ __forceinline__ void operator()() const {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -290,7 +298,7 @@ __device__ __forceinline__ void sell_row(const int32_t *__restrict__ sp, const i
     const int64_t c = __ldg(cp + (int64_t)t * 32);
     T xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
+    for (int q = 0; q < BC; ++q) xv[q] = ld_vec(x + c * BC + q);
     const T *v = vp + (int64_t)t * (BR * BC * 32);
 #pragma unroll
     for (int r = 0; r < BR; ++r)
@@ -306,7 +314,7 @@ __device__ __forceinline__ void sell_row(const int32_t *__restrict__ sp, const i
 // blocks of a lane at a time cost registers: 23^3 box AMG(BGS) 9.8 -> 10.1-12.1 ms.)
 template <int BR, int BC, typename T, class W>
 __device__ __forceinline__ void bsr_row(const int32_t *__restrict__ rp, const int32_t *__restrict__ col,
-                                        const T *__restrict__ val, const T *__restrict__ x, int64_t row, bool active,
+                                        const T *__restrict__ val, const T *x, int64_t row, bool active,
                                         int gl, int ls, W wait, T (&acc)[BR]) {
   int k = 0, hi = 0;
   if (active) {
@@ -326,7 +334,7 @@ __device__ __forceinline__ void bsr_row(const int32_t *__restrict__ rp, const in
     const int kn = k + (1 << ls);
     T xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
+    for (int q = 0; q < BC; ++q) xv[q] = ld_vec(x + c * BC + q);
     if (kn < hi) c = __ldg(col + kn);
 #pragma unroll
     for (int r = 0; r < BR; ++r)
@@ -441,7 +449,7 @@ __device__ __forceinline__ void cta_row(const int32_t *__restrict__ rp, const in
     const int64_t c = __ldg(col + k);
     T xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
+    for (int q = 0; q < BC; ++q) xv[q] = ld_vec(x + c * BC + q);
     T blk[BR * BC];
     ldg_block<BR * BC, T>(val + (int64_t)k * (BR * BC), blk);
 #pragma unroll
@@ -634,7 +642,7 @@ constexpr int kSellPad = 33;  // row pitch of the partial sums (bank conflicts)
 template <int BR, int BC, typename T, class W>
 __device__ __forceinline__ void sell_split_row(int64_t nbr, const int32_t *__restrict__ sp,
                                                const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
-                                               const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
+                                               const T *__restrict__ val, const T *x, int64_t slice,
                                                W wait, T (&acc)[BR]) {
   const int lane = threadIdx.x & 31, h = threadIdx.x >> 5, H = blockDim.x >> 5;
   const int64_t row = slice * 32 + lane;
@@ -658,7 +666,7 @@ __device__ __forceinline__ void sell_split_row(int64_t nbr, const int32_t *__res
   if (h < len) {
     T xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + c * BC + q);
+    for (int q = 0; q < BC; ++q) xv[q] = ld_vec(x + c * BC + q);
 #pragma unroll
     for (int r = 0; r < BR; ++r)
 #pragma unroll
@@ -669,7 +677,7 @@ __device__ __forceinline__ void sell_split_row(int64_t nbr, const int32_t *__res
     const int64_t ct = __ldg(cp + (int64_t)t * 32);
     T xv[BC];
 #pragma unroll
-    for (int q = 0; q < BC; ++q) xv[q] = __ldg(x + ct * BC + q);
+    for (int q = 0; q < BC; ++q) xv[q] = ld_vec(x + ct * BC + q);
     const T *v = vp + (int64_t)t * (BR * BC * 32);
 #pragma unroll
     for (int r = 0; r < BR; ++r)
@@ -681,7 +689,7 @@ __device__ __forceinline__ void sell_split_row(int64_t nbr, const int32_t *__res
 template <int BR, int BC, typename T, class W>
 __device__ __forceinline__ void sell_split_sums(int64_t nbr, const int32_t *__restrict__ sp,
                                                 const int32_t *__restrict__ rl, const int32_t *__restrict__ col,
-                                                const T *__restrict__ val, const T *__restrict__ x, int64_t slice,
+                                                const T *__restrict__ val, const T *x, int64_t slice,
                                                 W wait, T (*part)[BR][kSellPad]) {
   T acc[BR];
   sell_split_row<BR, BC, T>(nbr, sp, rl, col, val, x, slice, wait, acc);
@@ -924,11 +932,11 @@ __device__ __forceinline__ void d_spmv_rows(int64_t nbr, const int32_t *__restri
       const int64_t c = __ldg(cp + (int64_t)t * 32);
       double xv[BCT];
 #pragma unroll
-      for (int q = 0; q < B0; ++q) xv[q] = __ldg(x0 + c * B0 + q);
+      for (int q = 0; q < B0; ++q) xv[q] = ld_vec(x0 + c * B0 + q);
 #pragma unroll
-      for (int q = 0; q < B1; ++q) xv[B0 + q] = __ldg(x1 + c * B1 + q);
+      for (int q = 0; q < B1; ++q) xv[B0 + q] = ld_vec(x1 + c * B1 + q);
 #pragma unroll
-      for (int q = 0; q < B2; ++q) xv[B0 + B1 + q] = __ldg(x2 + c * B2 + q);
+      for (int q = 0; q < B2; ++q) xv[B0 + B1 + q] = ld_vec(x2 + c * B2 + q);
       const double *v = vp + (int64_t)t * (BR * BCT * 32);
 #pragma unroll
       for (int r = 0; r < BR; ++r)
@@ -1050,7 +1058,7 @@ __device__ __forceinline__ void gs_group_row(const int32_t *__restrict__ rp, con
     const int64_t c = __ldg(col + k);
     T xv[BR];
 #pragma unroll
-    for (int q = 0; q < BR; ++q) xv[q] = __ldg(x + c * BR + q);
+    for (int q = 0; q < BR; ++q) xv[q] = ld_vec(x + c * BR + q);
     T blk[BR * BR];
     ldg_block<BR * BR, T>(val + (int64_t)k * (BR * BR), blk);
 #pragma unroll

@@ -104,3 +104,23 @@ def test_device_products_equal_host_products(pc, kw):
                 assert np.abs(A.data - B.data).max() <= 1e-12 * np.abs(B.data).max()
     g.close()
     h.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32p"])
+@pytest.mark.parametrize("name,pc", [("box3-25", "amg_bgs"), ("box2-25", "simple"), ("box2-50", "bgs_amg")])
+def test_programmatic_launches_equal_ordinary_ones_on_split_sell(name, pc, prec):
+    """17,576 and 132,651 rows: the SELL-32 kernels with several threads a row
+    (alone and as fused products) and with one thread a row run as programmatic
+    dependent launches and still read their predecessors' results."""
+    s, kw = _system(name)
+    v = torch.from_numpy(np.random.default_rng(8).standard_normal(s.ndofs)).cuda()
+    b = torch.from_numpy(s.rhs).cuda()
+    with mfs.Solver(s, precond=pc, precision=prec, pdl=0, **kw) as off:
+        z, y = off.apply(v), off.matvec(v)
+        x, info, _ = off.solve(b, tol=1e-8)
+        for pdl in (1, -1):
+            with mfs.Solver(s, precond=pc, precision=prec, pdl=pdl, **kw) as on:
+                for _ in range(3):
+                    assert torch.equal(z, on.apply(v)) and torch.equal(y, on.matvec(v))
+                xp, ip, _ = on.solve(b, tol=1e-8)
+                assert ip["iters"] == info["iters"] and torch.equal(x, xp)

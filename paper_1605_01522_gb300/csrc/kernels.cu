@@ -2136,8 +2136,12 @@ void init() {
 // walks an average row in one step (8 blocks: 8 lanes), two steps for rows of
 // up to 32 blocks, more for longer ones.  In float64 the lanes' products
 // and sums bound these kernels (64 cycles a warp instruction): a 9-block row
-// of 3x3 blocks takes 9 warp instructions with 16 lanes, 24 with a warp.
+// of 3x3 blocks takes 9 warp instructions with 16 lanes, 24 with a warp.  A
+// row of over 1,024 blocks among short ones decides alone and takes all 32
+// (four rows of 4,000 blocks among 68,921 of 27, float64, 16 / 32 lanes: 3x3
+// 260 / 185 us, 1x1 80 / 74; of 1,051: 109 / 107 and 47 / 59).
 template <typename T> int bsr_ls(const Sell &A) {
+  if (A.longest > 1024) return 5;
   const double avg = (double)A.nnzb / (double)A.nbr;
   return avg <= 8.0 ? 3 : avg <= 32.0 ? 4 : 5;
 }

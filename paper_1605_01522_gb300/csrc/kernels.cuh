@@ -24,6 +24,7 @@ struct Sell {
   int unroll = 2;              // SELL-32: slots of a row in flight per thread (2, 4 or 8)
   int split = 1;               // SELL-32: threads per block row (1, or 2, 4, 8 with unroll 2)
   int br = 0, bc = 0;
+  int32_t longest = 0;         // blocks of the longest row
   int64_t nbr = 0, nbc = 0;
   int64_t nslices = 0, nslots = 0;
   int64_t nnzb = 0;            // true nonzero blocks (algorithmic size)

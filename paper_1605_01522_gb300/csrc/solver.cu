@@ -189,18 +189,33 @@ static int sell_split(int64_t nbr, double avg) {
 // 8,192 for short rows (prolongators, 4 blocks), which leave half the lanes
 // of a group idle (13,824 rows 13.4 / 13.5), from 49,152 for rows of over 32
 // blocks, which a lane walks longest (20,261 rows of 105 1x1 blocks 15.9 / 10.4
-// us a product, 68,921 of 114 16.2 / 20.3).  Rows of over 128 blocks and blocks
-// above 3x6 stay plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
+// us a product, 68,921 of 114 16.2 / 20.3).  Rows of over 128 blocks stay
+// plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
 // In batches the systems fill the GPU together, so the fewest instructions a
 // row win (96 systems of 1,089 rows float64: SELL-32 10.3 ms, plain BSR 14.4)
 // and 2 threads per row: 24 boxes of 729 to 15,625 rows 24.4 ms with 1 (tuned by
 // timing), 19.7 with 2, 19.4 with 4; 256 boxes of up to
 // 117,649 rows 626 ms with 4, 615 with 2).
-static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb) {
+// A few rows much longer than the mean keep plain BSR in both: the threads of
+// a SELL-32 row walk it alone, at up to 3 us a step of 3x3 blocks (four rows of
+// the given length among rows of 27, float64 product, SELL-32 / plain BSR:
+// 68,921 rows 3x3, 91 blocks 95 / 71 us, 4,000 3,052 / 185; 1x1, 283 34 / 39,
+// 539 46 / 42; 22,801 rows 1x1 of 9, 137 26 / 25, 521 43 / 29).
+static bool skewed(int br, int bc, double avg, int64_t longest) {
+  return longest * br * bc > 256 && (double)longest > 2.0 * avg;
+}
+static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb, int64_t longest) {
   const double avg = nbr ? (double)nnzb / (double)nbr : 0.0;
+  if (skewed(br, bc, avg, longest)) return 0;
   if (g_layout_tune == 1) return nbr >= 700 && br * bc <= 18 && avg <= 32.0 ? 2 : 0;
   if (br * bc > 18 || avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : avg <= 32.0 ? 16384 : 49152)) return 0;
   return sell_split(nbr, avg);
+}
+
+template <typename I> static int32_t longest_row(const std::vector<I> &rp) {
+  I m = 0;
+  for (size_t r = 1; r < rp.size(); ++r) m = std::max(m, rp[r] - rp[r - 1]);
+  return (int32_t)m;
 }
 
 static dev::Sell upload_layout(Arena &ar, const HBsr &A, bool want64, bool want32, int kind) {
@@ -210,6 +225,7 @@ static dev::Sell upload_layout(Arena &ar, const HBsr &A, bool want64, bool want3
   S.nbr = A.nbr;
   S.nbc = A.nbc;
   S.nnzb = A.nnzb();
+  S.longest = longest_row(A.rp);
   if (A.nbr == 0) return S;
   const int bs = A.br * A.bc;
   if (kind == 1) {
@@ -271,6 +287,7 @@ struct RawDev {
   int32_t *rp = nullptr, *ci = nullptr;
   double *v = nullptr;
   int br = 0, bc = 0;
+  int32_t longest = 0;  // blocks of the longest row
   int64_t nbr = 0, nbc = 0, nnzb = 0;
 };
 
@@ -283,6 +300,7 @@ static RawDev upload_raw(Arena &tmp, const HBsr &A, cudaStream_t st) {
   R.nnzb = A.nnzb();
   if (A.nnzb() > INT32_MAX) throw SetupError(MFS_ERR_INVALID, "matrix too large for 32-bit block offsets");
   std::vector<int32_t> rp(A.rp.begin(), A.rp.end());
+  R.longest = longest_row(rp);
   R.rp = tmp.alloc<int32_t>((int64_t)rp.size());
   R.ci = tmp.alloc<int32_t>(R.nnzb);
   R.v = tmp.alloc<double>(R.nnzb * R.br * R.bc);
@@ -311,6 +329,7 @@ static dev::Sell upload_layout_dev(Arena &ar, const RawDev *const *src, int nsrc
   S.nbr = A.nbr;
   S.nbc = A.nbc;
   S.nnzb = A.nnzb;
+  S.longest = A.longest;
   if (A.nbr == 0) return S;
   const int64_t bs = (int64_t)S.br * S.bc;
   if (kind == 1) {
@@ -459,7 +478,7 @@ static dev::Sell tune_keep(Arena &ar, dev::Sell &a, dev::Sell &b, int best) {
 
 static dev::Sell upload_sell(Arena &ar, const HBsr &A, bool want64, bool want32) {
   if (A.nbr < (g_layout_tune == 1 ? kTuneMinRowsBatch : kTuneMinRows)) {
-    const int h = small_layout(A.br, A.bc, A.nbr, A.nnzb());
+    const int h = small_layout(A.br, A.bc, A.nbr, A.nnzb(), longest_row(A.rp));
     dev::Sell S = upload_layout(ar, A, want64, want32, h ? 0 : 1);
     if (h) S.split = h;
     return S;
@@ -501,7 +520,7 @@ static dev::Sell upload_sell(Arena &ar, const HBsr &A, bool want64, bool want32)
 static dev::Sell upload_sell_dev(Arena &ar, const RawDev &A, bool want64, bool want32, cudaStream_t st) {
   const RawDev *src[1] = {&A};
   if (A.nbr < (g_layout_tune == 1 ? kTuneMinRowsBatch : kTuneMinRows)) {
-    const int h = small_layout(A.br, A.bc, A.nbr, A.nnzb);
+    const int h = small_layout(A.br, A.bc, A.nbr, A.nnzb, A.longest);
     dev::Sell S = upload_layout_dev(ar, src, 1, want64, want32, h ? 0 : 1, st);
     if (h) S.split = h;
     return S;

@@ -1,0 +1,76 @@
+"""Which row kernel the layout rules give a matrix, and its product against
+scipy, for matrices that no mesh of the repository has.  Needs a GB300.
+
+The handle takes the single-level Gauss-Seidel preconditioner (no hierarchy), so that
+any square matrix with a full diagonal can be given; a profiled solve names the
+kernels of the float64 products.  Bound of an entry of a product: (k + 64)
+2^-53 of |A| |x| with k terms in the longest row, what scipy's one chain may be
+off by (the kernels' shorter chains and the sums over lanes are off by less).
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+import scipy.sparse as sp
+
+from paper_1605_01522_gb300 import inputs, mfs
+
+pytestmark = pytest.mark.gpu
+
+
+def _banded(n, width, b, long_rows=0, length=0, seed=0):
+    """n block rows of `width` blocks around the diagonal (fewer at the ends),
+    `long_rows` of them with about `length` random columns more."""
+    rng = np.random.default_rng(seed)
+    off = np.arange(width) - width // 2
+    r = np.repeat(np.arange(n), width)
+    c = r + np.tile(off, n)
+    keep = (c >= 0) & (c < n)
+    r, c = r[keep], c[keep]
+    for k in range(long_rows):
+        row = (k * n) // max(1, long_rows) + 5
+        r = np.concatenate([r, np.full(length, row)])
+        c = np.concatenate([c, rng.choice(n, length, replace=False)])
+    key = np.unique(r.astype(np.int64) * n + c)
+    r, c = key // n, key % n
+    rp = np.searchsorted(r, np.arange(n + 1)).astype(np.int32)
+    v = rng.uniform(-1.0, 1.0, (len(r), b, b))
+    v[r == c] += 8.0 * np.eye(b)
+    return inputs.BSR(b, b, n, n, rp, c.astype(np.int32), v)
+
+
+def _system(m):
+    n = m.nbrows
+    f = inputs.Field("u", m.br, n, 3, np.zeros((n, 3)), "const")
+    rhs = np.random.default_rng(1).standard_normal(n * m.br)
+    return inputs.BlockSystem([f], {(0, 0): m}, rhs, name="banded")
+
+
+def _check(s, kernels, **kw):
+    """kernels: names that have to be among the solve's, or with a leading '-' must not be"""
+    A = sp.bmat([[s.blocks[(i, j)].to_scipy() if (i, j) in s.blocks else None for j in range(s.nfields)]
+                 for i in range(s.nfields)]).tocsr()
+    x = np.random.default_rng(2).standard_normal(s.ndofs)
+    with mfs.Solver(s, precond="bgs_gs", smoother="gs", profile=1, max_iters=2, **kw) as lib:
+        y = lib.matvec(torch.from_numpy(x).cuda()).cpu().numpy()
+        bound = (np.diff(A.indptr).max() + 64) * 2.0 ** -53
+        assert (np.abs(y - A @ x) <= bound * (abs(A) @ abs(x))).all()
+        lib.solve(torch.from_numpy(s.rhs).cuda(), tol=1e-8, check=False)
+        names = [r[0] for r in lib.kernel_detail()]
+    for k in kernels.split():
+        assert any(k.lstrip("-") in n for n in names) != k.startswith("-"), (k, names)
+
+
+@pytest.mark.parametrize("n,b,long_rows,length,tune,kernels", [
+    (20001, 1, 0, 0, 0, "spmv_sell_split<1x1,f64>"),            # even rows: SELL-32
+    (20001, 1, 3, 200, 0, "spmv_sell_split<1x1,f64>"),          # 200 blocks of one entry: still
+    (20001, 1, 3, 300, 0, "spmv_warp<1x1,f64> -sell_split"),    # 300: plain BSR
+    (20001, 3, 1, 60, 0, "spmv_warp<3x3,f64> -sell_split"),     # 3x3 blocks: from 57 on
+    (20001, 1, 2, 4000, 0, "spmv_warp<1x1,f64> -sell_split"),   # all 32 lanes
+    (1000, 2, 0, 0, 1, "spmv_sell_split<2x2,f64>"),             # batch setups
+    (1000, 2, 2, 300, 1, "spmv_warp<2x2,f64> -sell_split"),
+])
+def test_few_long_rows_keep_plain_bsr(n, b, long_rows, length, tune, kernels):
+    """The threads of a SELL-32 row walk it alone: one row of 4,000 3x3 blocks
+    among 68,921 of 27 took 3 ms there, 0.2 ms over the lanes of plain BSR."""
+    _check(_system(_banded(n, 27, b, long_rows, length)), kernels, layout_tune=tune)

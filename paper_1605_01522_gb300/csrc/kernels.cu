@@ -26,6 +26,8 @@ constexpr int kSellThreads = 64;
 // kCtaRowBlocks blocks per row take one CTA per row instead of one warp
 constexpr int64_t kCtaRowsMax = 4096;
 constexpr int64_t kCtaRowBlocks = 128;
+constexpr int64_t kCtaRowsMax64 = 1024;  // the same for float64 (cta_rows)
+constexpr int64_t kCtaRowBlocks64 = 768;
 constexpr int kGsCtaThreads = 1024;  // threads of the one-CTA Gauss-Seidel kernel for small levels
 LaunchHook *g_hook = nullptr;
 // > 0 while this thread's launches must bypass the process-wide hook
@@ -2152,11 +2154,17 @@ static unsigned bsr_threads(int64_t lanes) {
   while (t < (unsigned)kThreads && lanes > (int64_t)t * 152) t *= 2;
   return t;
 }
-// few, long rows: one CTA per row; not in float64, where the 8 warps' sums
-// over lanes take longer than the row (6x3 blocks, 184 a row: 22 us on 1,128
-// rows, 7 us with a warp per row)
+// Few, long rows: one CTA per row.  In float64 the 8 warps' sums over lanes
+// take longer than a row of a few hundred blocks (6x3 blocks, 184 a row, 1,128
+// rows: 22 us, 7 with a warp per row), so only very long rows of which there are
+// few (rows of 1x3 blocks of a call that also multiplies 29,791 3x3 rows, warp /
+// CTA: 20 rows of 600 blocks 47.9 / 47.6 us, of 1,000 50 / 47, of 3,000 66 / 50; 1,000
+// rows of 600 52 / 53, of 1,000 63 / 59; 2,000 rows 57 / 64 and 72 / 70, 4,000 66 / 80
+// and 82 / 89).
 template <typename T> bool cta_rows(const Sell &A) {
-  return sizeof(T) == 4 && A.kind == 1 && A.nbr <= kCtaRowsMax && A.nnzb >= kCtaRowBlocks * A.nbr;
+  constexpr int64_t rows = sizeof(T) == 4 ? kCtaRowsMax : kCtaRowsMax64;
+  constexpr int64_t blocks = sizeof(T) == 4 ? kCtaRowBlocks : kCtaRowBlocks64;
+  return A.kind == 1 && A.nbr <= rows && A.nnzb >= blocks * A.nbr;
 }
 
 template <typename T>

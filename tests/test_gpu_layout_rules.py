@@ -74,3 +74,29 @@ def test_few_long_rows_keep_plain_bsr(n, b, long_rows, length, tune, kernels):
     """The threads of a SELL-32 row walk it alone: one row of 4,000 3x3 blocks
     among 68,921 of 27 took 3 ms there, 0.2 ms over the lanes of plain BSR."""
     _check(_system(_banded(n, 27, b, long_rows, length)), kernels, layout_tune=tune)
+
+
+@pytest.mark.parametrize("rows,length,b,kernels", [
+    (4, 767, 3, "spmv_warp<1x3,f64>"),            # constraint rows: a warp each
+    (4, 768, 3, "spmv_cta<1x3,f64>"),             # a CTA each
+    (1024, 800, 1, "spmv_cta<1x1,f64>"),
+    (1025, 800, 1, "spmv_warp<1x1,f64>"),
+    (3, 5000, 6, "spmv_cta<1x6,f64>"),
+])
+def test_few_very_long_rows_take_a_cta_each(rows, length, b, kernels):
+    """Rows of multipliers against a large field; a warp walked 20 rows of
+    3,000 1x1 blocks in 46 us, a CTA a row in 35."""
+    n = 6000
+    rng = np.random.default_rng(3)
+    big = _banded(n, 9, b)
+    ci = np.concatenate([np.sort(rng.choice(n, length, replace=False)) for _ in range(rows)]).astype(np.int32)
+    A10 = inputs.BSR(1, b, rows, n, (np.arange(rows + 1) * length).astype(np.int32), ci,
+                     rng.uniform(-1.0, 1.0, (rows * length, 1, b)))
+    one = np.arange(rows + 1, dtype=np.int32)
+    A11 = inputs.BSR(1, 1, rows, rows, one, one[:-1].copy(), np.ones((rows, 1, 1)))
+    s = _system(big)
+    s.fields.append(inputs.Field("c", 1, rows, 3, np.zeros((rows, 3)), "const"))
+    s.blocks.update({(1, 0): A10, (1, 1): A11})
+    s.rhs = np.concatenate([s.rhs, np.ones(rows)])
+    # one product a row field would hide the kernel's name in a fused launch: batch setups keep them apart
+    _check(s, kernels, layout_tune=1)

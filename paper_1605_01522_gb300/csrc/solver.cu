@@ -190,7 +190,10 @@ static int sell_split(int64_t nbr, double avg) {
 // of a group idle (13,824 rows 13.4 / 13.5), from 49,152 for rows of over 32
 // blocks, which a lane walks longest (20,261 rows of 105 1x1 blocks 15.9 / 10.4
 // us a product, 68,921 of 114 16.2 / 20.3).  Rows of over 128 blocks stay
-// plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).
+// plain BSR (6x3 blocks, 184 a row, 5,997 rows: 102 / 20 us).  Blocks of all
+// sizes follow these lines (6x6, 27 a row, float64 product with 2, 4, 8 threads /
+// plain BSR: 17,576 rows 56, 58, 61 / 69 us, 68,921 rows 142, 142, 159 / 194; 12
+// such systems of 2,197 to 15,625 rows in a batch 12.7, 13.1, 17.2 / 15.9 ms).
 // In batches the systems fill the GPU together, so the fewest instructions a
 // row win (96 systems of 1,089 rows float64: SELL-32 10.3 ms, plain BSR 14.4)
 // and 2 threads per row: 24 boxes of 729 to 15,625 rows 24.4 ms with 1 (tuned by
@@ -207,8 +210,8 @@ static bool skewed(int br, int bc, double avg, int64_t longest) {
 static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb, int64_t longest) {
   const double avg = nbr ? (double)nnzb / (double)nbr : 0.0;
   if (skewed(br, bc, avg, longest)) return 0;
-  if (g_layout_tune == 1) return nbr >= 700 && br * bc <= 18 && avg <= 32.0 ? 2 : 0;
-  if (br * bc > 18 || avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : avg <= 32.0 ? 16384 : 49152)) return 0;
+  if (g_layout_tune == 1) return nbr >= 700 && avg <= 32.0 ? 2 : 0;
+  if (avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : avg <= 32.0 ? 16384 : 49152)) return 0;
   return sell_split(nbr, avg);
 }
 

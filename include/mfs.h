@@ -167,8 +167,10 @@ typedef struct {
   double gs_omega;                   /* MFS_GS: damping omega of the Gauss-Seidel update (0.79,
                                         the paper's DD(GS(0.79)), Sec. 7.1); 0 < omega < 2 */
   int rows_split;                    /* threads per block row of the float64 coupled matvec
-                                        (merged row layout): 0 (default) = timed at setup
-                                        among 1, 2, 4 and 8; or 1, 2, 4 to fix it */
+                                        (merged row layout): 0 (default) = 4, or 8 for up
+                                        to 2,500 rows of more than 16 blocks; from
+                                        131,072 rows on timed at setup among 1, 2 and
+                                        4; or 1, 2, 4 to fix it */
   int layout_tune;                   /* sparse layouts of matrices with >= 131,072 block rows
                                         (>= 2,048 with 1; smaller ones by a rule):
                                         0 (default) = the fastest of SELL-32 (2, 4 or 8

@@ -149,7 +149,7 @@ struct RowMerged {
   int nb = 0;      // number of merged column fields (2 or 3)
   int b[3] = {0, 0, 0};
   int64_t off[3] = {0, 0, 0};  // offset of each column field in the coupled vector
-  int split = 1;   // threads per block row (1, 2, 4 or 8), timed at setup
+  int split = 1;   // threads per block row (1, 2, 4 or 8), see tune_rows
 };
 // column fields of b[0], b[1][, b[2]] dofs per node, row field 0 of b[0], the others of one
 bool rows_supported(const int *b, int nb);

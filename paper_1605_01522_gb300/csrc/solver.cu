@@ -2243,12 +2243,21 @@ HBsr to_hbsr(const mfs_block &b) {
   return A;
 }
 
-// Threads per block row of the merged float64 matvec (1, 2, 4 or 8): timed
-// once per (column blocks, rows, blocks) and process, like the layouts.
+// Threads per block row of the merged float64 matvec.  Below kTuneMinRows rows by
+// a rule, as the layouts (single launches are timed to about 2 us, and the
+// choice changed the order of the sums from process to process): 4, which no
+// other count beats by more than the spread of its runs from 100 to 130,000
+// rows, alone and in batches (a call on the 3-field box with 1 / 2 / 4 / 8: 24^3
+// 43.0, 36.6, 32.3, 34.3 us, 47^3 143, 149, 141, 159; 16 boxes of 25^3 in a batch
+// 36.2, 34.5, 33.7, 35.1 ms), but 8 for up to 2,500 rows of more than 16 blocks,
+// whose few slices leave SMs idle (7^3 42.2, 36.4, 26.8, 26.3 us; 24 boxes of
+// 10^3 8.04, 6.35, 5.62, 5.53 ms).  From kTuneMinRows on 1, 2 and 4 are timed once
+// per (column blocks, rows, blocks) and process.
 static std::map<std::tuple<int, int, int, int64_t, int64_t>, int> g_tune_rows;
 
 static int tune_rows(const std::vector<dev::RowMerged> &R, int64_t n, cudaStream_t st) {
   const dev::Sell &A = R[0].M;
+  if (A.nbr < kTuneMinRows) return A.nbr <= 2500 && A.nnzb > 16 * A.nbr ? 8 : 4;
   const auto key = std::make_tuple(R[0].b[0], R[0].b[1], R[0].nb > 2 ? R[0].b[2] : 0, (int64_t)A.nbr, (int64_t)A.nnzb);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
@@ -2265,7 +2274,7 @@ static int tune_rows(const std::vector<dev::RowMerged> &R, int64_t n, cudaStream
   int best = 1;
   float tbest = 1e30f;
   std::vector<dev::RowMerged> T = R;
-  for (int split : {1, 2, 4, 8}) {
+  for (int split : {1, 2, 4}) {
     T[0].split = split;
     for (int rep = 0; rep < 4; ++rep) {
       MFS_CUDA(cudaEventRecord(e0, st));

@@ -110,3 +110,35 @@ def test_few_very_long_rows_take_a_cta_each(rows, length, b, kernels):
     s.rhs = np.concatenate([s.rhs, np.ones(rows)])
     # one product a row field would hide the kernel's name in a fused launch: batch setups keep them apart
     _check(s, kernels, layout_tune=1)
+
+
+@pytest.mark.parametrize("fields,n,width,same_as_four", [
+    ((3, 1, 1), 2, 2, True),
+    ((3, 1, 1), 33, 27, False),     # 8 threads a row; rows of one block, of 14 and of 27
+    ((3, 1), 2047, 27, False),
+    ((2, 1), 2500, 20, False),
+    ((2, 1), 2501, 20, True),
+    ((3, 1, 1), 1000, 12, True),    # short rows
+])
+def test_merged_rows_take_the_threads_of_the_rule(fields, n, width, same_as_four):
+    """The coupled matvec without rows_split, whose order of sums (and so its
+    bits) is the one with 4 threads a row or, for few long rows, with 8."""
+    rng = np.random.default_rng(n)
+    base = _banded(n, width, 1)
+    row = np.repeat(np.arange(n), np.diff(base.rowptr))
+    keep = (row % 13 != 12) | (base.colind == row)  # every 13th row: its diagonal alone
+    rp = np.searchsorted(row[keep], np.arange(n + 1)).astype(np.int32)
+    ci = base.colind[keep]
+    s = inputs.BlockSystem([], {}, rng.standard_normal(n * sum(fields)), name="banded")
+    for i, b in enumerate(fields):
+        s.fields.append(inputs.Field(f"f{i}", b, n, 3, np.zeros((n, 3)), "const"))
+        for j, c in enumerate(fields):
+            v = rng.uniform(-1.0, 1.0, (len(ci), b, c))
+            if i == j:
+                v[row[keep] == ci] += 8.0 * np.eye(b)
+            s.blocks[(i, j)] = inputs.BSR(b, c, n, n, rp, ci, v)
+    _check(s, "spmv_rows")
+    x = torch.from_numpy(rng.standard_normal(s.ndofs)).cuda()
+    kw = dict(precond="bgs_gs", smoother="gs")
+    with mfs.Solver(s, **kw) as a, mfs.Solver(s, rows_split=4, **kw) as b:
+        assert torch.equal(a.matvec(x), b.matvec(x)) == same_as_four

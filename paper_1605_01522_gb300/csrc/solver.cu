@@ -1340,7 +1340,10 @@ struct mfs_handle {
   bool own_stream = false;
   cudaEvent_t entry = nullptr;
   bool use_graphs = true;
-  std::vector<IterGraph> graphs;  // per Krylov index j
+  // per Krylov index j, with ordinary launches at j and with the automatic
+  // choice's programmatic ones at m + j: each solve replays the graphs of its
+  // own launch policy, whichever the handle's first solve had
+  std::vector<IterGraph> graphs;
   ~mfs_handle() {
     for (auto &g : graphs) g.release();
     if (hpin) g_pinned.put(hpin, kHostSlots * sizeof(double));
@@ -1416,10 +1419,10 @@ double dot_host(mfs_handle *h, const double *x, const double *y) {
   return h->hpin[kDotSlot];
 }
 
-// Capture body() once per Krylov index j into a CUDA graph and replay it:
-// one launch per GMRES iteration instead of one per kernel.
-template <typename F> void run_graph(mfs_handle *h, int j, F &&body, bool prof) {
-  IterGraph &g = h->graphs[j];
+// Capture body() once per Krylov index and launch policy (slot) into a CUDA
+// graph and replay it: one launch per GMRES iteration instead of one per kernel.
+template <typename F> void run_graph(mfs_handle *h, int slot, F &&body, bool prof) {
+  IterGraph &g = h->graphs[slot];
   if (!g.exec) {
     if (prof) {
       h->prof->cap_events = &g.events;
@@ -1531,13 +1534,14 @@ static std::atomic<int> g_solves_running{0};
 // call runs alone (16 concurrent solves of small systems measured 2 % slower
 // with them).
 struct SolvePhase {
+  bool programmatic = false;  // the automatic choice took programmatic launches
   explicit SolvePhase(const mfs_handle *h) {
     const bool alone = ++g_solves_running == 1;
     const int p = h->prm.pdl;
     unsigned g = 0, g64 = 0;
     if (p == 1) g = g64 = ~0u;
     else if (p > 1) g = g64 = (unsigned)p;
-    else if (p == -1 && alone) g = ~0u, g64 = 160u;
+    else if (p == -1 && alone) g = ~0u, g64 = 160u, programmatic = true;
     dev::set_pdl(g, g64);
   }
   ~SolvePhase() {
@@ -1597,7 +1601,7 @@ int fgmres(mfs_handle *h, const double *b, double *x, double tol, mfs_info *info
       MFS_CUDA(cudaMemcpyAsync(hpb[j & 1], hdb[j & 1], 136 * sizeof(double), cudaMemcpyDeviceToHost, s));
       dev::pdl_break();
     };
-    if (h->use_graphs) run_graph(h, j, body, prof);
+    if (h->use_graphs) run_graph(h, phase.programmatic ? m + j : j, body, prof);
     else body();
     MFS_CUDA(cudaEventRecord(h->iter_ev[j & 1], s));
     dev::pdl_break();
@@ -2634,7 +2638,7 @@ void upload_precond(mfs_handle *h, Arena &mat, Precond<T> &P, const std::map<std
 // GMRES workspace of a handle.
 void alloc_solver_work(mfs_handle *h) {
   h->m = h->prm.restart;
-  h->graphs.assign(h->m, IterGraph());
+  h->graphs.assign(2 * (size_t)h->m, IterGraph());
   h->nblk = dev::mdot_blocks(h->n, h->prm.layout_tune == 1);
   h->V = h->ar.zeros<double>((int64_t)(h->m + 1) * h->n);
   h->Z = h->ar.zeros<double>((int64_t)h->m * h->n);

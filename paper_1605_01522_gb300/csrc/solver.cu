@@ -168,8 +168,9 @@ static PinnedCache &g_pinned = *new PinnedCache();
 // layouts made their setups longer.
 constexpr int64_t kTuneMinRows = 131072;
 constexpr int64_t kTuneMinRowsBatch = 16384;
-// mfs_params.layout_tune of the setup running on this thread
+// mfs_params.layout_tune and vcycle_tail of the setup running on this thread
 static thread_local int g_layout_tune = 0;
+static thread_local bool g_vcycle_tail = false;
 
 // Threads per block row of a SELL-32 matrix of nbr rows of avg blocks: 8 for
 // long rows, 4 for short ones, halved while the matrix would take more than
@@ -210,7 +211,9 @@ static bool skewed(int br, int bc, double avg, int64_t longest) {
 static int small_layout(int br, int bc, int64_t nbr, int64_t nnzb, int64_t longest) {
   const double avg = nbr ? (double)nnzb / (double)nbr : 0.0;
   if (skewed(br, bc, avg, longest)) return 0;
-  if (g_layout_tune == 1) return nbr >= 700 && avg <= 32.0 ? 2 : 0;
+  // with V-cycle tails, which read plain BSR, rows up to what a tail of scalar
+  // float rows can hold (48 KB, five vectors) stay there
+  if (g_layout_tune == 1) return nbr >= (g_vcycle_tail ? 2458 : 700) && avg <= 32.0 ? 2 : 0;
   if (avg > 128.0 || nbr < (avg <= 12.0 ? 8192 : avg <= 32.0 ? 16384 : 49152)) return 0;
   return sell_split(nbr, avg);
 }
@@ -2722,10 +2725,16 @@ int mfs_setup(const mfs_block *blocks, int nblocks, const mfs_field *fields, int
   }
   const double t0 = now_ms();
   std::unique_ptr<mfs_handle> h(new mfs_handle());
-  struct TuneMode {  // the layout tuning mode of this setup, for this thread
-    explicit TuneMode(int m) { g_layout_tune = m; }
-    ~TuneMode() { g_layout_tune = 0; }
-  } tune_mode(p.layout_tune);
+  struct TuneMode {  // what the layouts of this setup depend on, for this thread
+    explicit TuneMode(const mfs_params &q) {
+      g_layout_tune = q.layout_tune;
+      g_vcycle_tail = q.vcycle_tail != 0;
+    }
+    ~TuneMode() {
+      g_layout_tune = 0;
+      g_vcycle_tail = false;
+    }
+  } tune_mode(p);
   try {
     h->prm = p;
     h->nf = nfields;

@@ -14,6 +14,7 @@ torch = pytest.importorskip("torch")
 import scipy.sparse as sp
 
 from paper_1605_01522_gb300 import inputs, mfs
+from tests.oracle_from_lib import oracle_preconditioner
 
 pytestmark = pytest.mark.gpu
 
@@ -142,3 +143,21 @@ def test_merged_rows_take_the_threads_of_the_rule(fields, n, width, same_as_four
     kw = dict(precond="bgs_gs", smoother="gs")
     with mfs.Solver(s, **kw) as a, mfs.Solver(s, rows_split=4, **kw) as b:
         assert torch.equal(a.matvec(x), b.matvec(x)) == same_as_four
+
+
+@pytest.mark.parametrize("ne,prec,tol", [(30, "fp64", 1e-12), (33, "fp64", 1e-12), (47, "fp32p", 2e-3)])
+def test_batch_setups_keep_the_vcycle_tail(ne, prec, tol):
+    """Scalar levels of 700 rows and more that fit the one-CTA tail (961 and
+    1,156 rows in float64, 2,304 in float32) take it in batch setups too.
+    Bounds: the other application tests' for float64; in float32 a rounding of
+    6e-8 from each of 16 steps, times the condition of the coarse matrices
+    (1,784 for elasticity)."""
+    s = inputs.thermo_elastic_2d(ne=ne)
+    v = np.random.default_rng(3).standard_normal(s.ndofs)
+    with mfs.Solver(s, precond="bgs_amg", precision=prec, layout_tune=1, vcycle_tail=1, profile=1, max_iters=2,
+                    max_levels=2, coarse_max=0) as lib:
+        z = lib.apply(torch.from_numpy(v).cuda()).cpu().numpy()
+        zr = oracle_preconditioner(lib, s)(v)
+        assert np.abs(z - zr).max() <= tol * np.abs(zr).max()
+        lib.solve(torch.from_numpy(s.rhs).cuda(), tol=1e-8, check=False)
+        assert any(r[0] == "vcycle_tail" for r in lib.kernel_detail())

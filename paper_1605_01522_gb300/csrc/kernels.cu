@@ -2561,7 +2561,7 @@ int mdot_blocks(int64_t n, bool batch) {
   }
   int best = 1;
   double tbest = 1e300;
-  for (int ctas = 1; ctas <= 6; ++ctas) {  // CTAs per SM
+  for (int ctas = 1; ctas <= kMdotBlocksMax / 152; ++ctas) {  // CTAs per SM
     const int64_t per = (tiles + 152 * ctas - 1) / (152 * ctas);
     const int64_t nblk = (tiles + per - 1) / per;
     if (per > 1 && ctas < (per > 2 ? 3 : 2)) continue;

@@ -245,6 +245,7 @@ void scale_convert_dev(double *v, const double *inv, TO *out, int64_t n, cudaStr
 // partial: k * nblk doubles of scratch, nblk = mdot_blocks(n) (batch: for a
 // system solved together with others); out: device memory; cnt: a device
 // counter that is 0 between passes.
+constexpr int kMdotBlocksMax = 6 * 152;  // mdot_blocks never gives more (760 reached, at 194,560 entries)
 int mdot_blocks(int64_t n, bool batch = false);
 // out[q] = V_q . w; with out null only partial[q*nblk+b], for a later
 // reduce_partials.  One row with cnt given is reduced by the pass itself

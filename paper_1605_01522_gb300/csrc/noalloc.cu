@@ -20,9 +20,10 @@ void set_last_error(const char *msg);  // thread-local detail behind mfs_last_er
 
 namespace {
 
-// MFS_DOT_NOALLOC_PARTIALS partial sums (one per reduction block; the
-// chunking of dev::mdot_blocks never asks for more than 608) plus the result.
+// MFS_DOT_NOALLOC_PARTIALS partial sums (one per reduction block of
+// dev::mdot_blocks) plus the result.
 constexpr int kPartials = MFS_DOT_NOALLOC_PARTIALS;
+static_assert(kPartials >= mfs::dev::kMdotBlocksMax, "a partial sum per reduction block");
 static __device__ __align__(256) double g_dot_scratch[kPartials + 32];
 
 constexpr int kMaxDevices = 64;

@@ -74,6 +74,18 @@ def test_dot_at_tile_edges(n):
     assert abs(d - float(np.dot(x, y))) <= 1e-13 * float(np.abs(x) @ np.abs(y))
 
 
+def test_dot_with_the_most_partial_sums_then_fewer():
+    """194,560 entries are 760 tiles of 256, one CTA each: the largest number of
+    partial sums of any length.  A shorter call afterwards reads only its own."""
+    rng = np.random.default_rng(11)
+    for n in (194560, 194559, 194560 - 256 + 3, 5037, 194560, 77):
+        x, y = rng.standard_normal(n), rng.standard_normal(n)
+        xd, yd = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+        d = mfs.dot_noalloc(xd, yd)
+        assert abs(d - float(np.dot(x, y))) <= 1e-13 * float(np.abs(x) @ np.abs(y))
+        assert d == mfs.dot_noalloc(xd, yd)
+
+
 @pytest.mark.parametrize("restart", [5, 33, 60])
 @pytest.mark.parametrize("tune", [0, 1])
 def test_basis_stays_orthogonal_at_every_row_count(restart, tune):

@@ -175,28 +175,32 @@ def reduce_timing(elapsed, steps, world, dist=None, device=None):
     return world * steps / elapsed, elapsed
 
 
-def kernel_source_digest(kernel):
-    """sha256 of the device source of a kernel variant family (its __global__
-    function and the row helper it calls), to tell whether stored ncu
+def kernel_source_digest(kernel, src=None):
+    """sha256 of the device source of a kernel variant family (its traits
+    struct and the row helpers it calls), to tell whether stored ncu
     counters still describe the current code."""
     import hashlib
     import re
-    src = open(os.path.join(ROOT, "paper_1605_01522_gb300", "csrc", "kernels.cu")).read()
-    fn = {"smooth_sell": ["sell_row", "d_smooth"], "spmv_sell": ["sell_row", "d_spmv"],
-          "smooth_sell4": ["sell_row", "d_smooth"], "spmv_sell4": ["sell_row", "d_spmv"],
-          "smooth_sell8": ["sell_row", "d_smooth"], "spmv_sell8": ["sell_row", "d_spmv"],
-          "spmv_rows": ["d_spmv_rows"], "smooth_warp": ["bsr_row", "group_sum"],
-          "spmv_warp": ["bsr_row", "group_sum"]}.get(kernel.split("<")[0])
-    if fn:
-        fn = fn + ["k_solo"]  # the single-system kernel wrapper every launch goes through
+    if src is None:
+        src = open(os.path.join(ROOT, "paper_1605_01522_gb300", "csrc", "kernels.cu")).read()
+    sell = {"smooth": ["sell_row", "d_smooth", "KSmoothSell"], "spmv": ["sell_row", "d_spmv", "KSpmvSell"]}
+    split = ["sell_split_row", "sell_split_sums", "sell_split_entry"]
+    fn = {"smooth_sell": sell["smooth"], "spmv_sell": sell["spmv"],
+          "smooth_sell4": sell["smooth"], "spmv_sell4": sell["spmv"],
+          "smooth_sell8": sell["smooth"], "spmv_sell8": sell["spmv"],
+          "smooth_sell_split": split + ["KSmoothSellSplit"], "spmv_sell_split": split + ["KSpmvSellSplit"],
+          "spmv_rows": ["d_spmv_rows", "KSpmvRows"], "smooth_warp": ["bsr_row", "group_sum", "KSmoothWarp"],
+          "spmv_warp": ["bsr_row", "group_sum", "KSpmvWarp"]}.get(kernel.split("<")[0])
     if not fn:
         return None
+    fn = fn + ["ld_vec", "k_solo"]  # loads of vectors; the single-system wrapper every launch goes through
     h = hashlib.sha256()
     for f in fn:
-        m = re.search(r"(template <[^>]*>\s*)?(__device__|__global__)[^{;]*\b" + f + r"\(", src)
+        head = r"struct " + f + r" \{" if f[0] == "K" else r"(__device__|__global__)[^{;]*\b" + f + r"\("
+        m = re.search(r"(template <[^>]*>\s*)?" + head, src)
         if not m:
             return None
-        depth, i = 0, src.index("{", m.end())
+        depth, i = 0, src.index("{", m.end() - 1)
         for j in range(i, len(src)):
             depth += {"{": 1, "}": -1}.get(src[j], 0)
             if depth == 0:

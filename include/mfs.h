@@ -171,21 +171,22 @@ typedef struct {
                                         to 2,500 rows of more than 16 blocks; from
                                         131,072 rows on timed at setup among 1, 2 and
                                         4; or 1, 2, 4 to fix it */
-  int layout_tune;                   /* sparse layouts of matrices with >= 131,072 block rows
-                                        (>= 2,048 with 1; smaller ones by a rule):
-                                        0 (default) = the fastest of SELL-32 (2, 4 or 8
-                                        slots in flight, or 2, 4 or 8 threads per
-                                        row) and one warp per row, each timed
-                                        alone (best for one solve at a time: a mid-size
-                                        matrix cannot fill the GPU by itself); 1 = the same
-                                        with one thread per row, and one warp per row only
-                                        for rows of >= 32 blocks
-                                        (best when many systems run together,
-                                        mfs_solve_batch, where the GPU is full and
-                                        throughput counts) */
+  int layout_tune;                   /* sparse layouts.  0 (default), for one solve at a
+                                        time: below 131,072 block rows by a rule on rows
+                                        and blocks per row (SELL-32 with 2, 4 or 8 threads
+                                        per row, or plain BSR with 8, 16 or 32 lanes per
+                                        row), from there on the fastest of these and of
+                                        SELL-32 with one thread per row, timed at setup.
+                                        1, for many systems together (mfs_solve_batch),
+                                        which fill the GPU: below 16,384 rows by a rule
+                                        (SELL-32 with 2 threads per row from 700 rows of at
+                                        most 32 blocks on - 2,458 rows with vcycle_tail -
+                                        else plain BSR), from there on timed among SELL-32
+                                        with one thread per row and, for rows of >= 32
+                                        blocks, plain BSR */
   int vcycle_tail;                   /* 1: a single-field V-cycle whose level above the
-                                        coarsest is small (<= 48 KB of vectors, one warp per
-                                        block row, explicit coarse inverse) runs that level
+                                        coarsest is small (<= 48 KB of vectors, plain-BSR
+                                        layout, explicit coarse inverse) runs that level
                                         and the coarse solve as ONE single-CTA launch (same
                                         arithmetic, bit for bit); 0 (default): one launch per
                                         step (Algorithm 1 as written) - on GB300 the one-SM
@@ -362,7 +363,7 @@ int mfs_kernel_stats(struct mfs_handle *h, double *out, int cap, int reset);
  * kernel variant and size, sorted by summed time: [cls*100000 + sig, rows,
  * launches, ms, algorithmic bytes, algorithmic flops], where for SpMV (cls 0) and smoothing
  * (cls 1) sig = layout*1000 + br*100 + bc*10 + (float64 ? 1 : 0) with layout
- * 0 = SELL-32, 1 = warp-per-row BSR, 2 = merged coupled rows, 3 = SELL-32 with
+ * 0 = SELL-32, 1 = plain BSR (8 to 32 lanes per row), 2 = merged coupled rows, 3 = SELL-32 with
  * 4 slots in flight, 8 = SELL-32 with several threads per row (the layout autotuner's choices), and rows = block rows; for the other
  * classes sig is a kernel id and rows the vector length.  Returns the number
  * of rows written (cap = length of out).  Cleared by mfs_kernel_stats with

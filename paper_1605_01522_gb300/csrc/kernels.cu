@@ -241,7 +241,7 @@ template <typename T> double matrix_bytes(const Sell &A) {
 // 16, 8-byte ones when a multiple of 8, else one load per entry.  Block k
 // starts k * N * sizeof(T) bytes into a value array that starts on a 16-byte
 // boundary (every value array is its own allocation; the setup checks it), so
-// every vector is aligned.  Fewer, wider loads keep the load queue of one-warp-per-row
+// every vector is aligned.  Fewer, wider loads keep the load queue of the plain-BSR
 // kernels from filling (6x6 float blocks: 9 loads instead of 36).
 template <int N, typename T>
 __device__ __forceinline__ void ldg_block(const T *__restrict__ p, T (&o)[N]) {
@@ -1889,8 +1889,8 @@ struct KGemvAdd {
 // zero, residual, restriction, the coarsest solve through the explicit
 // inverse, prolongation and post-smoothing, separated by __syncthreads
 // instead of kernel boundaries.  Every step reduces a row exactly as the
-// separate launches do (one warp per block row, lanes striding over the
-// row's blocks, the same xor butterfly; the inverse applied in float64), so
+// separate launches do (bsr_ls lanes per block row striding over its blocks,
+// the same halving sums; the inverse applied in float64), so
 // the result is the one of the step-by-step V-cycle bit for bit.
 constexpr int kTailThreads = 1024;
 constexpr int kTailMaxSteps = 8;

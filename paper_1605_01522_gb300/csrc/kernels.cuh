@@ -16,9 +16,9 @@ namespace mfs {
 namespace dev {
 
 struct Sell {
-  int kind = 0;                // 0: SELL-32, one thread per block row;
-                               // 1: plain BSR, one warp per block row (long rows /
-                               //    few rows: restriction, coarse levels); then sp is
+  int kind = 0;                // 0: SELL-32, `split` threads per block row;
+                               // 1: plain BSR, 8, 16 or 32 lanes per block row (long
+                               //    rows / few rows: restriction, coarse levels); then sp is
                                //    the row pointer, col the block columns and the
                                //    values are contiguous per block (br*bc, row-major)
   int unroll = 2;              // SELL-32: slots of a row in flight per thread (2, 4 or 8)
@@ -43,8 +43,8 @@ struct Sell {
 enum KernelClass { K_SPMV = 0, K_SMOOTH = 1, K_VECTOR = 2, K_COARSE = 3, K_ARNOLDI = 4, K_NCLASS = 5 };
 // sig identifies the kernel variant: for SpMV / smoothing
 // layout*1000 + br*100 + bc*10 + (float64 ? 1 : 0) with layout 0 SELL-32,
-// 1 warp BSR, 2 merged rows, 3 SELL-32 with 4 slots in flight, 4 / 5 / 6 the
-// Gauss-Seidel colour kernels on SELL-32 / warp BSR / SELL-32 x4, 7 one CTA per
+// 1 plain BSR, 2 merged rows, 3 SELL-32 with 4 slots in flight, 4 / 5 / 6 the
+// Gauss-Seidel colour kernels on SELL-32 / plain BSR / SELL-32 x4, 7 one CTA per
 // BSR row, 8 SELL-32 with several threads per row, 10 / 11 a sum of bc products in one
 // launch (plain BSR / SELL-32); otherwise a small id.
 // rows = block rows (sparse kernels) or vector length.

@@ -11,8 +11,9 @@
 //    then the two joining phases;
 //  * tentative prolongator: one warp per aggregate, two-pass Gram-Schmidt;
 //  * lambda_max: 10 power iterations; smoothing, transpose and Galerkin
-//    products with a warp-per-row block SpGEMM (hash set for the pattern,
-//    then a sequential sweep over the row's products for the values).
+//    products with a warp-per-row block SpGEMM (hash set for the pattern;
+//    values: the entries of A's row one after another, the products of one of
+//    them by the lanes at the same time).
 #include "setup_gpu.h"
 
 #include <cuda_runtime.h>

@@ -199,7 +199,10 @@ static int sell_split(int64_t nbr, double avg) {
 // row win (96 systems of 1,089 rows float64: SELL-32 10.3 ms, plain BSR 14.4)
 // and 2 threads per row: 24 boxes of 729 to 15,625 rows 24.4 ms with 1 (tuned by
 // timing), 19.7 with 2, 19.4 with 4; 256 boxes of up to
-// 117,649 rows 626 ms with 4, 615 with 2).
+// 117,649 rows 626 ms with 4, 615 with 2).  The line at 700 rows is a mean of
+// cases (plain BSR / SELL-32: 96 2D systems float64 of 441 rows 8.3, 7.2 ms, 729
+// 10.6, 8.1, float32 7.2, 6.7 and 8.0, 7.5; 24 boxes float32 of 512 rows 4.3, 4.5, 1,000
+// 5.4, 5.5, float64 5.1, 5.2 and 6.8, 6.1).
 // A few rows much longer than the mean keep plain BSR in both: the threads of
 // a SELL-32 row walk it alone, at up to 3 us a step of 3x3 blocks (four rows of
 // the given length among rows of 27, float64 product, SELL-32 / plain BSR:
@@ -235,7 +238,7 @@ static dev::Sell upload_layout(Arena &ar, const HBsr &A, bool want64, bool want3
   if (A.nbr == 0) return S;
   const int bs = A.br * A.bc;
   if (kind == 1) {
-    // plain BSR, one warp per block row
+    // plain BSR
     if (A.nnzb() > INT32_MAX) throw SetupError(MFS_ERR_INVALID, "matrix too large for 32-bit block offsets");
     S.kind = 1;
     std::vector<int32_t> rp(A.rp.begin(), A.rp.end());
@@ -430,7 +433,7 @@ static std::mutex g_tune_mu;
 static std::map<std::tuple<int, int, int64_t, int64_t, int>, int> g_tune;
 
 // Layout candidates of the autotuner: 0 SELL-32 with 2 slots in flight,
-// 1 with 4, 2 plain BSR with one warp per row, 3 SELL-32 with 8 slots in
+// 1 with 4, 2 plain BSR (8 to 32 lanes per row), 3 SELL-32 with 8 slots in
 // flight (only for blocks of at most 3 entries, whose rows are short on bytes),
 // 4, 5, 6 SELL-32 with 2, 4, 8 threads per row (the one of sell_split; tuning
 // for batches leaves them out, other systems fill the GPU there).
@@ -443,7 +446,7 @@ static int tune_pick(const dev::Sell &a, const dev::Sell &b, bool want32, cudaSt
   float t[kTuneCands];
   t[0] = want32 ? time_spmv<float>(a, st) : time_spmv<double>(a, st);
   t[1] = want32 ? time_spmv<float>(a4, st) : time_spmv<double>(a4, st);
-  // throughput tuning leaves the one-warp-per-row layout out for short rows
+  // throughput tuning leaves the plain-BSR layout out for short rows
   // (fewer blocks than lanes: idle lanes; SELL-32 moves more rows per
   // microsecond when the GPU is full) but keeps it for long rows such as a
   // restriction's, which one thread per row would walk serially
@@ -879,8 +882,11 @@ template <typename T> struct Precond {
     FL<T> &f = g.lv[l][i], &c = g.lv[l + 1][i];
     dev::RowTerm<T> t{&f.R, r};
     bool done = false;
-    // (long restrictions are not launch bound: 5,997 rows of 184 6x3 blocks
-    // took 32 us this way, 26 + 7 us as two launches; 1x1 14 and 9 + 7)
+    // up to 1.5 M entries: longer restrictions are not launch bound, and the fused
+    // kernel's registers cost more there than the launch (whole solves of 30
+    // iterations with the limit at 0 / 1.5 M / none: 46^3 box BGS f32 17.61, 17.30,
+    // 17.32 ms; 23^3 f64 11.01, 10.74, 10.75; 50^3 AMG(BGS) 27.87, 27.83, 28.51; 2-field
+    // 36^3 SIMPLE f64 13.29, 13.26, 13.47)
     const bool small = f.R.nnzb * f.R.br * f.R.bc <= 1500000;
     if (smoothed && small && smoother != MFS_GS && fusable(&t, 1)) {
       dev::RowOut<T> o;

@@ -161,3 +161,38 @@ def test_batch_setups_keep_the_vcycle_tail(ne, prec, tol):
         assert np.abs(z - zr).max() <= tol * np.abs(zr).max()
         lib.solve(torch.from_numpy(s.rhs).cuda(), tol=1e-8, check=False)
         assert any(r[0] == "vcycle_tail" for r in lib.kernel_detail())
+
+
+def _coupled(n, width, nf, wide=None, wide_width=0):
+    """nf scalar fields of n nodes, all pairs coupled; block `wide` has rows of wide_width."""
+    s = inputs.BlockSystem([], {}, np.random.default_rng(4).standard_normal(n * nf), name="coupled")
+    for i in range(nf):
+        s.fields.append(inputs.Field(f"f{i}", 1, n, 3, np.zeros((n, 3)), "const"))
+        for j in range(nf):
+            s.blocks[(i, j)] = _banded(n, wide_width if (i, j) == wide else width, 1, seed=10 * i + j)
+    return s
+
+
+@pytest.mark.parametrize("n,width,nf,wide,wide_width,kernels", [
+    (333, 9, 4, None, 0, "spmv_terms_bsr<1x4,f64>"),                             # four products: one launch
+    (333, 9, 5, None, 0, "spmv_warp<1x1,f64> spmv_terms_bsr<1x4,f64>"),          # five: one by one (the sweep's four fused)
+    (20001, 27, 2, None, 0, "spmv_terms_sell<1x2,f64> -spmv_warp"),
+    (20001, 27, 2, (0, 1), 161, "spmv_warp<1x1,f64> spmv_sell_split<1x1,f64> spmv_terms_sell<1x2,f64>"),  # two layouts in row 0
+])
+def test_products_of_a_row_are_fused_where_the_layouts_allow_it(n, width, nf, wide, wide_width, kernels):
+    _check(_coupled(n, width, nf, wide, wide_width), kernels)
+
+
+@pytest.mark.parametrize("length,kernels", [(767, "spmv_terms_bsr<1x2,f64> -spmv_cta"), (768, "spmv_cta<1x3,f64> -terms")])
+def test_cta_rows_stay_out_of_fused_products(length, kernels):
+    n, rows = 6000, 5
+    rng = np.random.default_rng(6)
+    ci = np.concatenate([np.sort(rng.choice(n, length, replace=False)) for _ in range(rows)]).astype(np.int32)
+    one = np.arange(rows + 1, dtype=np.int32)
+    s = _system(_banded(n, 9, 3))
+    s.fields.append(inputs.Field("c", 1, rows, 3, np.zeros((rows, 3)), "const"))
+    s.blocks[(1, 0)] = inputs.BSR(1, 3, rows, n, (np.arange(rows + 1) * length).astype(np.int32), ci,
+                                  rng.uniform(-1.0, 1.0, (rows * length, 1, 3)))
+    s.blocks[(1, 1)] = inputs.BSR(1, 1, rows, rows, one, one[:-1].copy(), np.ones((rows, 1, 1)))
+    s.rhs = np.concatenate([s.rhs, np.ones(rows)])
+    _check(s, kernels, bgs_order="fwd")
